@@ -31,6 +31,7 @@
 #include "gq_internal.cuh"
 #include "gq_dfl.cuh"
 #include "gq_math.cuh"
+#include "gq_eval.cuh"
 
 namespace {
 
@@ -51,34 +52,6 @@ constexpr int kBinN = 64;   // binomial table C(n, k), n, k < 64
 // M2L applied at QBX order (List 3 far to centres).  Read with warp-uniform
 // indices, so constant-cache broadcasts serve it.
 __constant__ double c_pascal[GQ_MAX_PQBX + 1][33];
-
-struct EvalView {
-    RootInfo R;
-    int P, Q, kernel;
-    const int *blev, *bix, *biy, *bparent;
-    const int4 *bchild;
-    const int *src_beg, *src_end;
-    const int *ctr_beg, *ctr_end, *pt_beg, *pt_end;
-    const int *sub_src, *sub_tgt;
-    const double2 *s_xy;
-    const double2 *str;
-    const double2 *sc_xy;
-    const double *sc_r;
-    const double2 *sp_xy;
-    const int *loff[6];
-    const int *lidx[6];
-    const double *binom;   // [kBinN][kBinN]
-    const int *qc;         // per-centre QBX order (sorted centres) or nullptr: all use Q
-    const double *logt;    // GqLogTable
-    const unsigned int *qexp;   // largest biased exponent of the S strengths (k_strengths)
-    int nwork_ctr;              // boxes owning centres (batched items)
-};
-
-__device__ __forceinline__ double box_rho(const RootInfo &R, int l) { return ldexp(R.H, -l); }
-__device__ __forceinline__ double2 box_centre(const RootInfo &R, int l, int ix, int iy) {
-    double h = ldexp(R.H, -l);
-    return make_double2(R.lo_x + (double)(2 * ix + 1) * h, R.lo_y + (double)(2 * iy + 1) * h);
-}
 
 __device__ __forceinline__ double2 shfl2(double2 v, int src, int width) {
     return make_double2(__shfl_sync(0xffffffffu, v.x, src, width), __shfl_sync(0xffffffffu, v.y, src, width));
@@ -372,198 +345,6 @@ __global__ void k_p2l(EvalView E, int nwork, const int *__restrict__ work, doubl
 }
 
 // ------------------------------------------------------------------ Stages 3, 5a, 6a: direct near field
-// One block per target box; the box's List 1, 3 close and 4 close source
-// ranges are flattened into shared memory; each warp takes one target and its
-// lanes stride over the flattened sources.
-constexpr int kNearThreads = 128;
-constexpr int kNearRanges = 256;
-
-struct NearRanges {
-    int beg[kNearRanges];
-    int pre[kNearRanges + 1];
-    int n;
-};
-
-__device__ int block_excl_scan_128(int v, int *wsum) {
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[w] = x;
-    __syncthreads();
-    int off = 0;
-    for (int i = 0; i < w; ++i) off += wsum[i];
-    __syncthreads();
-    return off + x - v;
-}
-
-// load entries [e0, e0 + kNearRanges) of the concatenated lists U, WC, XC of box b
-__device__ void load_ranges(const EvalView &E, int b, int e0, int ne, NearRanges &R, int *wsum) {
-    int n0 = E.loff[0][b + 1] - E.loff[0][b], n2 = E.loff[2][b + 1] - E.loff[2][b];
-    int cnt = min(kNearRanges, ne - e0);
-    int lens[2] = {0, 0};
-    for (int r = 0; r < 2; ++r) {
-        int i = threadIdx.x * 2 + r;
-        if (i < cnt) {
-            int e = e0 + i, d;
-            if (e < n0) d = E.lidx[0][E.loff[0][b] + e];
-            else if (e < n0 + n2) d = E.lidx[2][E.loff[2][b] + e - n0];
-            else d = E.lidx[4][E.loff[4][b] + e - n0 - n2];
-            R.beg[i] = E.src_beg[d];
-            lens[r] = E.src_end[d] - E.src_beg[d];
-        }
-    }
-    int pre = block_excl_scan_128(lens[0] + lens[1], wsum);
-    if (threadIdx.x * 2 < kNearRanges) R.pre[threadIdx.x * 2] = pre;
-    if (threadIdx.x * 2 + 1 < kNearRanges) R.pre[threadIdx.x * 2 + 1] = pre + lens[0];
-    if (threadIdx.x == kNearThreads - 1) R.pre[kNearRanges] = pre + lens[0] + lens[1];
-    if (threadIdx.x == 0) R.n = cnt;
-    __syncthreads();
-}
-
-// Warp reduce-scatter of NV values per lane: at each of the five butterfly
-// steps a lane keeps one half of its values, sends the other half to its
-// partner and adds what it receives, so a warp spends about NV adds instead of
-// 5 NV.  Afterwards lane L holds the warp sums of the original entries
-// base .. base + cnt - 1 in v[0 .. cnt) (cnt may be 0; for NV <= 32 it is 0 or 1).
-template <int N, int O, class V, class Add, class Shfl>
-__device__ __forceinline__ void rs_step(V *v, int lane, V zero, Add add, Shfl shfl, int &base, int &cnt) {
-    constexpr int H = (N + 1) / 2;
-    const bool up = (lane & O) != 0;
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-        V x = v[i], y = (i + H < N) ? v[i + H < N ? i + H : 0] : zero;
-        V send = up ? x : y, keep = up ? y : x;
-        v[i] = add(keep, shfl(send, O));
-    }
-    if (up) {
-        base += H;
-        cnt -= H;
-    } else if (cnt > H) {
-        cnt = H;
-    }
-}
-
-template <int NV, class V, class Add, class Shfl>
-__device__ __forceinline__ void warp_reduce_scatter(V (&v)[NV], V zero, int lane, Add add, Shfl shfl, int &base,
-                                                    int &cnt) {
-    constexpr int H1 = (NV + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2, H4 = (H3 + 1) / 2;
-    base = 0;
-    cnt = NV;
-    rs_step<NV, 16>(v, lane, zero, add, shfl, base, cnt);
-    rs_step<H1, 8>(v, lane, zero, add, shfl, base, cnt);
-    rs_step<H2, 4>(v, lane, zero, add, shfl, base, cnt);
-    rs_step<H3, 2>(v, lane, zero, add, shfl, base, cnt);
-    rs_step<H4, 1>(v, lane, zero, add, shfl, base, cnt);
-    if (cnt < 0) cnt = 0;
-}
-
-// QBX coefficients at centres: S: Q_0 = sum q log|w|, Q_m = -(1/m) sum q (r/w)^m;
-// D: Q_m = sum (d/w) (r/w)^m, with w = y - c.  One warp per centre, lanes
-// stride over the sources; the coefficients are summed by a reduce-scatter.
-template <int QQ, int KERNEL>
-__global__ void __launch_bounds__(kNearThreads) k_near_centres(EvalView E, int nwork, const int *__restrict__ work,
-                                                                double2 *__restrict__ Qout) {
-    __shared__ NearRanges R;
-    __shared__ int wsum[kNearThreads / 32];
-    __shared__ double lt[kGqLogN];
-    for (int i = threadIdx.x; i < kGqLogN; i += kNearThreads) lt[i] = E.logt[i];
-    // FP32 strengths are rebased to the largest one: q = qf * 2^(qe - 1023)
-    const int qe = KERNEL == GQ_D ? 1023 : (int)*E.qexp;
-    const double qscale = gq_pow2_biased(qe);
-    int b = work[blockIdx.x];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int ne = (E.loff[0][b + 1] - E.loff[0][b]) + (E.loff[2][b + 1] - E.loff[2][b]) + (E.loff[4][b + 1] - E.loff[4][b]);
-    int cb = E.ctr_beg[b], ce = E.ctr_end[b];
-    bool single = ne <= kNearRanges;
-    if (single) load_ranges(E, b, 0, ne, R, wsum);
-    for (int c0 = cb; c0 < ce; c0 += kNearThreads / 32) {
-        int c = c0 + w;
-        bool valid = c < ce;
-        double2 cz = valid ? E.sc_xy[c] : make_double2(0.0, 0.0);
-        double rc = valid ? E.sc_r[c] : 1.0;
-        const int qc = (valid && E.qc) ? E.qc[c] : QQ;
-        double2 acc[QQ + 1];
-#pragma unroll
-        for (int m = 0; m <= QQ; ++m) acc[m] = make_double2(0.0, 0.0);
-        float acc0f = 0.0f;   // S: FP32 tails of the logarithms, strengths rebased by qe
-        for (int e0 = 0; e0 < ne; e0 += kNearRanges) {
-            if (!single) {
-                __syncthreads();
-                load_ranges(E, b, e0, ne, R, wsum);
-            }
-            int T = R.pre[R.n];
-            if (valid) {
-                int r = 0;
-                for (int v = lane; v < T; v += 32) {
-                    while (R.pre[r + 1] <= v) ++r;
-                    int s = R.beg[r] + (v - R.pre[r]);
-                    double2 y = E.s_xy[s], st = E.str[s];
-                    double wx = y.x - cz.x, wy = y.y - cz.y;
-                    double n2 = wx * wx + wy * wy;
-                    double inv = gq_rcp(n2);
-                    double2 winv = make_double2(wx * inv, -wy * inv);    // 1/w (D only)
-                    double2 u;                                            // r/w
-                    if (KERNEL == GQ_D) {
-                        u = make_double2(rc * winv.x, rc * winv.y);
-                    } else {
-                        double ir = rc * inv;
-                        u = make_double2(wx * ir, -wy * ir);
-                    }
-                    if (KERNEL == GQ_D) {
-                        double2 t = cmul(st, winv);
-                        acc[0] = cadd(acc[0], t);
-#pragma unroll
-                        for (int m = 1; m < QQ; ++m) {
-                            if (m > qc) break;
-                            t = cmul(t, u);
-                            acc[m] = cadd(acc[m], t);
-                        }
-                        // last term: a multiply-add into the sum (t is not needed again)
-                        if (qc >= QQ) acc[QQ] = cfma(t, u, acc[QQ]);
-                    } else {
-                        float tail;
-                        acc[0].x = fma(st.x, gq_log_half_split(n2, lt, tail), acc[0].x);
-                        acc0f = fmaf(gq_f32_rebased(st.x, qe), tail, acc0f);
-                        double2 t = make_double2(st.x * u.x, st.x * u.y);
-                        acc[1] = cadd(acc[1], t);
-#pragma unroll
-                        for (int m = 2; m < QQ; ++m) {
-                            if (m > qc) break;
-                            t = cmul(t, u);
-                            acc[m] = cadd(acc[m], t);
-                        }
-                        if (QQ >= 2 && qc >= QQ) acc[QQ] = cfma(t, u, acc[QQ]);
-                    }
-                }
-            }
-        }
-        if (KERNEL != GQ_D) acc[0].x = fma((double)acc0f, qscale, acc[0].x);
-        double vals[2 * (QQ + 1)];
-#pragma unroll
-        for (int m = 0; m <= QQ; ++m) {
-            vals[2 * m] = acc[m].x;
-            vals[2 * m + 1] = acc[m].y;
-        }
-        int base, cnt;
-        warp_reduce_scatter(vals, 0.0, lane, [](double a, double x) { return a + x; },
-                            [](double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }, base, cnt);
-        if (valid) {
-            double *dst = reinterpret_cast<double *>(Qout + (size_t)c * (QQ + 1));
-#pragma unroll
-            for (int j = 0; j < (2 * (QQ + 1) + 31) / 32; ++j)
-                if (j < cnt) {
-                    int i = base + j, m = i >> 1;
-                    double x = vals[j];
-                    if (KERNEL != GQ_D && m >= 1) x *= -1.0 / m;
-                    dst[i] = x;
-                }
-        }
-    }
-}
-
 // potential at point targets: S: sum q log|t - y| (coincident sources skipped), D: Re sum d/(y - t)
 // Body for target box b (a block of kNearThreads); lt holds the log table
 // (S) in shared memory, loaded by the caller.
@@ -1214,7 +995,6 @@ struct SplitView {
     const float4 *lvl;   // per level l: [2l] = (rho, 1/rho), [2l+1] = (log rho, 1/rho^2)
     const float *logt;   // GqDflLogTable
     float H;             // root half-width (a power of two)
-    float fb;            // sources with |w|^2 < fb r^2 are taken in FP64 (fb >= 1)
     bool near_pt;        // point-target pairs closer than 1/8 of the box half-width in FP64
 };
 
@@ -1266,182 +1046,6 @@ __global__ void k_to_dfl4(long long n, const double2 *__restrict__ in, float4 *_
     if (j >= n) return;
     dfl a = dfl_from_double(in[j].x), b = dfl_from_double(in[j].y);
     out[j] = make_float4(a.hi, a.lo, b.hi, b.lo);
-}
-
-// Direct interactions to centres with every per-pair step in FP32 pairs: the
-// difference w = y - c, 1/|w|^2, 1/w, r/w, the power recurrence and the lane
-// sums of the coefficients.  For S the logarithm is split as
-// log|w| = log r + (1/2) log(|w|^2 / r^2), so that the pair logarithm sees
-// arguments >= 1 of modest size and log r enters once per centre in FP64.
-// Sources inside the expansion disk (|r/w| > 1) would amplify the rounding by
-// |r/w|^m and are taken in FP64, as in the FP32 tier.
-template <int QQ, int KERNEL>
-__global__ void __launch_bounds__(kNearThreads) k_near_centres_split(EvalView E, SplitView X, int nwork,
-                                                                      const int *__restrict__ work,
-                                                                      double2 *__restrict__ Qout) {
-    __shared__ NearRangesF R;
-    __shared__ int wsum[kNearThreads / 32];
-    __shared__ float lt[KERNEL == GQ_D ? 1 : 384];
-    __shared__ double lt64[KERNEL == GQ_D ? 1 : kGqLogN];
-    if (KERNEL != GQ_D) {
-        for (int i = threadIdx.x; i < 384; i += kNearThreads) lt[i] = X.logt[i];
-        for (int i = threadIdx.x; i < kGqLogN; i += kNearThreads) lt64[i] = E.logt[i];
-    }
-    int b = work[blockIdx.x];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int ne = (E.loff[0][b + 1] - E.loff[0][b]) + (E.loff[2][b + 1] - E.loff[2][b]) + (E.loff[4][b + 1] - E.loff[4][b]);
-    int cb = E.ctr_beg[b], ce = E.ctr_end[b];
-    double2 zb = box_centre(E.R, E.blev[b], E.bix[b], E.biy[b]);
-    bool single = ne <= kNearRanges;
-    if (single) load_ranges_f(E, b, zb, 0, ne, R, wsum);
-    for (int c0 = cb; c0 < ce; c0 += kNearThreads / 32) {
-        int c = c0 + w;
-        bool valid = c < ce;
-        float4 c4 = valid ? X.c_rel[c] : make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 r4 = valid ? X.c_r[c] : make_float4(1.f, 0.f, 1.f, 0.f);
-        dfl rc{r4.x, r4.y}, irc2{r4.z, r4.w};
-        float rc2 = r4.x * r4.x;
-        const int qc = (valid && E.qc) ? E.qc[c] : QQ;
-        double2 czd = valid ? E.sc_xy[c] : make_double2(0.0, 0.0);
-        double rcd = valid ? E.sc_r[c] : 1.0;
-        dflc acc[QQ + 1];
-        double2 acc64[QQ + 1];   // sources inside the expansion disk: FP64
-#pragma unroll
-        for (int m = 0; m <= QQ; ++m) {
-            acc[m] = dflc{dfl{0.f, 0.f}, dfl{0.f, 0.f}};
-            acc64[m] = make_double2(0.0, 0.0);
-        }
-        dfl acc_log{0.f, 0.f}, acc_str{0.f, 0.f};   // S: sum of st log(|w|^2/r^2), sum of st
-        bool used64 = false;
-        for (int e0 = 0; e0 < ne; e0 += kNearRanges) {
-            if (!single) {
-                __syncthreads();
-                load_ranges_f(E, b, zb, e0, ne, R, wsum);
-            }
-            int T = R.pre[R.n];
-            if (valid) {
-                int r = 0, rcur = -1;
-                dfl ex{0.f, 0.f}, ey{0.f, 0.f};   // source-box offset minus the centre
-                for (int v = lane; v < T; v += 32) {
-                    while (R.pre[r + 1] <= v) ++r;
-                    if (r != rcur) {
-                        float2 o = R.off[r];
-                        ex = dfl_add_f(dfl{-c4.x, -c4.y}, o.x);
-                        ey = dfl_add_f(dfl{-c4.z, -c4.w}, o.y);
-                        rcur = r;
-                    }
-                    int s = R.beg[r] + (v - R.pre[r]);
-                    float4 y4 = X.s_rel[s];
-                    dfl wx = dfl_add(dfl{y4.x, y4.y}, ex), wy = dfl_add(dfl{y4.z, y4.w}, ey);
-                    dfl n2 = dfl_add(dfl_sqr(wx), dfl_sqr(wy));
-                    if (n2.hi < rc2 * X.fb) {
-                        used64 = true;
-                        double2 yd = E.s_xy[s], sd = E.str[s];
-                        double dx = yd.x - czd.x, dy = yd.y - czd.y;
-                        double d2 = dx * dx + dy * dy, dinv = 1.0 / d2;
-                        double2 wi = make_double2(dx * dinv, -dy * dinv);
-                        double2 uu = make_double2(rcd * wi.x, rcd * wi.y);
-                        if (KERNEL == GQ_D) {
-                            double2 t = cmul(sd, wi);
-                            acc64[0] = cadd(acc64[0], t);
-#pragma unroll
-                            for (int m = 1; m <= QQ; ++m) {
-                                t = cmul(t, uu);
-                                acc64[m] = cadd(acc64[m], t);
-                            }
-                        } else {
-                            acc64[0].x += sd.x * gq_log_half(d2, lt64);
-                            double2 t = make_double2(sd.x * uu.x, sd.x * uu.y);
-                            acc64[1] = cadd(acc64[1], t);
-#pragma unroll
-                            for (int m = 2; m <= QQ; ++m) {
-                                t = cmul(t, uu);
-                                acc64[m] = cadd(acc64[m], t);
-                            }
-                        }
-                        continue;
-                    }
-                    float4 s4 = X.str[s];
-                    dfl inv = dfl_rcp(n2);
-                    dflc winv{dfl_mul(wx, inv), dfl_neg(dfl_mul(wy, inv))};
-                    dflc u{dfl_mul(rc, winv.re), dfl_mul(rc, winv.im)};
-                    dflc t;
-                    if (KERNEL == GQ_D) {
-                        t = dflc_mul(dflc{dfl{s4.x, s4.y}, dfl{s4.z, s4.w}}, winv);
-                        dflc_acc(acc[0], t);
-#pragma unroll
-                        for (int m = 1; m <= QQ; ++m) {
-                            if (m > qc) break;
-                            t = dflc_mul(t, u);
-                            dflc_acc(acc[m], t);
-                        }
-                    } else {
-                        dfl st{s4.x, s4.y};
-                        dfl lg = dfl_log(dfl_mul(n2, irc2), lt, lt + 128, lt + 256);
-                        dfl_acc(acc_log, dfl_mul(st, lg));
-                        dfl_acc(acc_str, st);
-                        t = dflc{dfl_mul(st, u.re), dfl_mul(st, u.im)};
-                        dflc_acc(acc[1], t);
-#pragma unroll
-                        for (int m = 2; m <= QQ; ++m) {
-                            if (m > qc) break;
-                            t = dflc_mul(t, u);
-                            dflc_acc(acc[m], t);
-                        }
-                    }
-                }
-            }
-        }
-        // warp sums by reduce-scatter: pairs in the FP32 pipe, the FP64 part only
-        // where a lane of the warp used it.  For S the constant term is folded
-        // first: Q_0 = (1/2) sum st log(|w|^2/r^2) + log r sum st.
-        const bool any64 = __any_sync(0xffffffffu, used64);
-        if (KERNEL != GQ_D) {
-            dfl lrc = dfl_log(dfl_sqr(rc), lt, lt + 128, lt + 256);   // log r^2
-            acc[0].re = dfl_add(dfl_mul_f(dfl_two_sum(acc_log.hi, acc_log.lo), 0.5f),
-                                dfl_mul(dfl_two_sum(acc_str.hi, acc_str.lo), dfl{0.5f * lrc.hi, 0.5f * lrc.lo}));
-        }
-        dfl vals[2 * (QQ + 1)];
-#pragma unroll
-        for (int m = 0; m <= QQ; ++m) {
-            vals[2 * m] = dfl_two_sum(acc[m].re.hi, acc[m].re.lo);
-            vals[2 * m + 1] = dfl_two_sum(acc[m].im.hi, acc[m].im.lo);
-        }
-        int base, cnt;
-        warp_reduce_scatter(vals, dfl{0.f, 0.f}, lane, [](dfl a, dfl x) { return dfl_add(a, x); },
-                            [](dfl x, int o) {
-                                return dfl{__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
-                            },
-                            base, cnt);
-        constexpr int NJ = (2 * (QQ + 1) + 31) / 32;
-        double v64[NJ];
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) v64[j] = 0.0;
-        if (any64) {
-            double d64[2 * (QQ + 1)];
-#pragma unroll
-            for (int m = 0; m <= QQ; ++m) {
-                d64[2 * m] = acc64[m].x;
-                d64[2 * m + 1] = acc64[m].y;
-            }
-            int b2, c2;
-            warp_reduce_scatter(d64, 0.0, lane, [](double a, double x) { return a + x; },
-                                [](double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }, b2, c2);
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) v64[j] = d64[j];
-        }
-        if (valid) {
-            double *dst = reinterpret_cast<double *>(Qout + (size_t)c * (QQ + 1));
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                if (j < cnt) {
-                    int i = base + j, m = i >> 1;
-                    double x = dfl_to_double(vals[j]) + v64[j];
-                    if (KERNEL != GQ_D && m >= 1) x *= -1.0 / m;
-                    dst[i] = x;
-                }
-        }
-    }
 }
 
 // Potential at point targets from List 1 sources, every pair step in FP32
@@ -1910,25 +1514,6 @@ __global__ void k_m2l_split(EvalView E, SplitView X, int nwork, const int *__res
 }
 
 template <int QQ>
-void launch_near_centres_split(gq_ctx *ctx, const EvalView &E, const SplitView &X, int nwork, const int *work,
-                               double2 *Q) {
-    auto kd = k_near_centres_split<QQ, GQ_D>;
-    auto ks = k_near_centres_split<QQ, GQ_S>;
-    GQ_LAUNCH(ctx, (E.kernel == GQ_D ? kd : ks), nwork, kNearThreads, 0, E, X, nwork, work, Q);
-}
-
-void dispatch_near_centres_split(gq_ctx *ctx, const EvalView &E, const SplitView &X, int nwork, const int *work,
-                                 double2 *Q) {
-    switch (E.Q) {
-#define GQ_CASE(v) case v: launch_near_centres_split<v>(ctx, E, X, nwork, work, Q); break;
-        GQ_CASE(1) GQ_CASE(2) GQ_CASE(3) GQ_CASE(4) GQ_CASE(5) GQ_CASE(6) GQ_CASE(7) GQ_CASE(8)
-        GQ_CASE(9) GQ_CASE(10) GQ_CASE(11) GQ_CASE(12) GQ_CASE(13) GQ_CASE(14) GQ_CASE(15) GQ_CASE(16)
-#undef GQ_CASE
-        default: throw gq_error{GQ_ERR_INVALID, "p_qbx out of range"};
-    }
-}
-
-template <int QQ>
 void launch_near_centres_f32(gq_ctx *ctx, const EvalView &E, const MixedView &X, int nwork, const int *work,
                              double2 *Q) {
     auto kd = k_near_centres_f32<QQ, GQ_D>;
@@ -2086,26 +1671,6 @@ void dispatch_near_centres_multi(gq_ctx *ctx, const EvalView &E, int nwork, cons
     }
 }
 
-template <int QQ>
-void launch_near_centres(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Q) {
-    auto kd = k_near_centres<QQ, GQ_D>;
-    auto ks = k_near_centres<QQ, GQ_S>;
-    if (E.kernel == GQ_D)
-        GQ_LAUNCH(ctx, kd, nwork, kNearThreads, 0, E, nwork, work, Q);
-    else
-        GQ_LAUNCH(ctx, ks, nwork, kNearThreads, 0, E, nwork, work, Q);
-}
-
-void dispatch_near_centres(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Q) {
-    switch (E.Q) {
-#define GQ_CASE(v) case v: launch_near_centres<v>(ctx, E, nwork, work, Q); break;
-        GQ_CASE(1) GQ_CASE(2) GQ_CASE(3) GQ_CASE(4) GQ_CASE(5) GQ_CASE(6) GQ_CASE(7) GQ_CASE(8)
-        GQ_CASE(9) GQ_CASE(10) GQ_CASE(11) GQ_CASE(12) GQ_CASE(13) GQ_CASE(14) GQ_CASE(15) GQ_CASE(16)
-#undef GQ_CASE
-        default: throw gq_error{GQ_ERR_INVALID, "p_qbx out of range"};
-    }
-}
-
 __global__ void k_tgt_ptpos(int npt, const int *__restrict__ pt_perm, int *__restrict__ out) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < npt) out[pt_perm[j]] = j;
@@ -2229,6 +1794,7 @@ __global__ void __launch_bounds__(kNearThreads) k_batch_persistent(const BatchGe
 // map of its current build.
 struct ConstTables {
     const double *logt = nullptr;     // GqLogTable
+    const FxLogTable *fxlog = nullptr;   // fixed-point logarithm
     const float *dlogt = nullptr;     // GqDflLogTable
     const double *binom = nullptr;    // [64][64]
     const double2 *dtab = nullptr;    // [121][32] delta^-k
@@ -2332,6 +1898,9 @@ static const ConstTables &const_tables(int dev) {
     gq_dfl_log_table_host(&DT);
     ConstTables C;
     C.logt = upload_const((const double *)&LT, kGqLogN);
+    FxLogTable FT;
+    fx_log_table_host(&FT);
+    C.fxlog = upload_const(&FT, 1);
     C.dlogt = upload_const((const float *)&DT, 384);
     C.binom = upload_const(bn.data(), bn.size());
     C.dtab = upload_const(dt.data(), dt.size());
@@ -2425,6 +1994,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     E.binom = T.binom;
     E.qc = g->has_qc ? (const int *)g->q_ctr.p : nullptr;
     E.logt = T.logt;
+    E.fxlog = T.fxlog;
 
     g->strength.alloc(g->nsrc);
     E.str = g->strength;
@@ -2534,10 +2104,6 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         }
         SX.s_rel = g->s_rel2; SX.str = g->str2; SX.c_rel = g->c_rel2; SX.c_r = g->c_r2; SX.p_rel = g->p_rel2;
         SX.M = g->M2; SX.lvl = g->lvl2; SX.logt = T.dlogt; SX.H = (float)g->root.H;
-        // only the sources inside the disk go to FP64: widening that region to |r/w| > 1/2
-        // lowered the added D rounding on a small grid from 1.6e-13 to 1.45e-13 only, and
-        // its divergent FP64 lanes tripled the kernel time
-        SX.fb = 1.0f;
         SX.near_pt = g->prm.eps < 1e-10;
     }
     mark(S_STR, st);
@@ -2548,8 +2114,9 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     mark(N_BEG, s2);
     if (g->n_ctr_boxes && !fmm_only) {
         if (f32) dispatch_near_centres_f32(&ctx2, E, X, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
-        else if (split) dispatch_near_centres_split(&ctx2, E, SX, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
-        else if (!qn_pre) dispatch_near_centres(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
+        // the FP32-pair tier too: fixed point is faster than pairs (1.05 M nodes, q = 4: 3.18 ms in pairs) and
+        // closer to 64 bits
+        else if (!qn_pre || split) gq_near_centres_fx(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
     }
     mark(N_CTR, s2);
     if (g->n_pt_boxes && !at_base && !fmm_only) {
@@ -2776,6 +2343,7 @@ static void gq_batch_geom_view(gq_geom *g, int kernel, BatchGeomDev &out) {
     E.binom = T.binom;
     E.qc = g->has_qc ? (const int *)g->q_ctr.p : nullptr;
     E.logt = T.logt;
+    E.fxlog = T.fxlog;
     E.nwork_ctr = g->n_ctr_boxes;
     out.E = E;
     out.ctr_boxes = g->ctr_boxes;
@@ -2997,6 +2565,7 @@ void gq_eval_multi(gq_geom *g, int kernel, int nd, const double *const *dens, do
     E.binom = T.binom;
     E.qc = g->has_qc ? (const int *)g->q_ctr.p : nullptr;
     E.logt = T.logt;
+    E.fxlog = T.fxlog;
     int d0 = 0;
     for (; d0 + 4 <= nd; d0 += 4)
         dispatch_near_centres_multi<4>(ctx, E, g->n_ctr_boxes, g->ctr_boxes, g->strm.p + d0 * sstride, sstride,
@@ -3037,10 +2606,12 @@ constexpr size_t kNaBinom = 0;                  // [64][64] doubles, 32 KiB
 constexpr size_t kNaDtab = 32768;               // [121][32] double2, 61,952 B
 constexpr size_t kNaLogtab = 98304;             // [121] doubles
 constexpr size_t kNaLogt = 99328;               // GqLogTable
+constexpr size_t kNaFxlog = 123904;             // FxLogTable, 6,144 B
 constexpr size_t kNaM2M = 131072;               // [4][kTN][kTN] double2, 61,504 B
 constexpr size_t kNaL2L = 196608;               // [4][kTN][kTN] double2
 constexpr size_t kNaQexp = 261888;              // one unsigned int, written by every call
-static_assert(kNaLogt + sizeof(double) * kGqLogN <= kNaM2M, "log table overlaps the M2M matrices");
+static_assert(kNaLogt + sizeof(double) * kGqLogN <= kNaFxlog, "log tables overlap");
+static_assert(kNaFxlog + sizeof(FxLogTable) <= kNaM2M, "log table overlaps the M2M matrices");
 static_assert(kNaL2L + sizeof(double2) * 4 * kTN * kTN <= kNaQexp, "tables exceed their region");
 static_assert(kNaQexp + 256 <= kNoAllocTableBytes, "exponent slot outside the table region");
 
@@ -3079,6 +2650,9 @@ NoAllocDevice &noalloc_setup(int dev) {
     GqLogTable LT;
     gq_log_table_host(&LT);
     GQ_CUDA(cudaMemcpy(base + kNaLogt, &LT, sizeof(LT), cudaMemcpyHostToDevice));
+    FxLogTable FT;
+    fx_log_table_host(&FT);
+    GQ_CUDA(cudaMemcpy(base + kNaFxlog, &FT, sizeof(FT), cudaMemcpyHostToDevice));
     GQ_CUDA(cudaMemcpy(base + kNaM2M, tm.data(), sizeof(double2) * tm.size(), cudaMemcpyHostToDevice));
     GQ_CUDA(cudaMemcpy(base + kNaL2L, tl.data(), sizeof(double2) * tl.size(), cudaMemcpyHostToDevice));
     std::vector<double> pc((GQ_MAX_PQBX + 1) * 33, 0.0);
@@ -3142,6 +2716,7 @@ void gq_eval_noalloc_impl(gq_geom *g, int kernel, const double *dens_dev, double
     E.binom = binom;
     E.qc = g->has_qc ? (const int *)g->q_ctr.p : nullptr;
     E.logt = (const double *)(D.base + kNaLogt);
+    E.fxlog = (const FxLogTable *)(D.base + kNaFxlog);
     E.qexp = qexp;
 
     // the array keeps the previous call's contents: clear the accumulators
@@ -3179,7 +2754,7 @@ void gq_eval_noalloc_impl(gq_geom *g, int kernel, const double *dens_dev, double
         GQ_LAUNCH(ctx, k_l2l_t, gq_blocks(e - s, 128 / P1), (128 / P1) * P1, 0, E, s, e, tl2l, L);
     }
     // the direct part writes the coefficients, the List 3 far and local parts add to them
-    if (g->n_ctr_boxes) dispatch_near_centres(ctx, E, g->n_ctr_boxes, g->ctr_boxes, Qc);
+    if (g->n_ctr_boxes) gq_near_centres_fx(ctx, E, g->n_ctr_boxes, g->ctr_boxes, Qc);
     if (g->n_pt_boxes) {
         auto kd = k_near_points<GQ_D>;
         auto ks = k_near_points<GQ_S>;

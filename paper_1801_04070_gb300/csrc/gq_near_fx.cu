@@ -1,0 +1,364 @@
+// gq_near_fx.cu -- Stages 3, 5a, 6a: the direct sums to the QBX centres with the
+// powers, logarithms and sums in 64-bit fixed point (gq_fix.cuh).
+//
+// S: Q_0 = sum q log|w|, Q_m = -(1/m) sum q (r/w)^m; D: Q_m = sum (d/w) (r/w)^m,
+// w = y - c.  In FP64 this sum issues 62 FP64 instructions a pair at q = 8 and
+// holds the FP64 pipe 88 % busy; here four are left (w and |w|^2), and 1/|w|^2,
+// r/w, log|w|, the power recurrence and the sums run on the integer pipes.  At
+// q = 8 a pair of a warp issues 440 instructions, about 110 of them 32 x 32 bit
+// multiply-adds of four cycles, which with the other work of that pipe bound
+// the kernel.  1.05 M quadrature nodes, 142.5 M pairs, S, q = 8: 17.06 ms -> 3.3 ms;
+// D on 0.14 M nodes: 2.59 -> 0.53 ms; q = 5 on one curve: 0.35 -> 0.14 ms.
+//
+// Formats (bits behind the binary point in brackets): u = r/w [62], t_m = q u^m
+// [60] with the strengths scaled to at most 1/2, products rounded at 2^-60.
+// |u| <= 1 when no source is inside the centre's disk; the loop records the
+// smallest |w|^2, and a centre that meets |u| > 1 + 1/64 is summed again with
+// the smallest |w| as its radius (the sums are then scaled by (r/|w|)^m).
+// Sums: 12 terms a lane (tiles of 384 sources), |t_m| < 0.65, stay below 2^63;
+// the warp's sum is taken at 2^-60 (2^-55 if the lanes' sums are that large).  Error against long double sums on the nodes
+// of a starfish grid (272 sources, q = 8, root mean square, in units of the
+// strength scale), FP64 form -> this: Q_0 2^-46.3 -> 2^-50.9, Q_1 2^-48.7 ->
+// 2^-53.0, Q_4 2^-50.9 -> 2^-52.1, Q_8 2^-50.5 -> 2^-51.5.
+//
+// The scale is that of the tile's own strengths, so that a strong source far away
+// costs a centre no accuracy.  Strengths that have none (infinite, NaN, exponents
+// near the ends of the range) and sources at the centre itself go through near_centre_slow, an
+// FP64 sum order by order with the arithmetic's own infinities and NaN.
+#include <math.h>
+
+#include "gq_eval.cuh"
+#include "gq_math.cuh"
+
+namespace {
+
+constexpr int kFxTile = 384;
+constexpr int kFxWarps = kNearThreads / 32;
+
+// a source's strength: S (h, l) [62]; D (re.h, re.l, im.h, im.l) [60], split at bit 30
+template <int KERNEL> struct FxStr { typedef int2 T; };
+template <> struct FxStr<GQ_D> { typedef int4 T; };
+
+// -1/m
+__constant__ double c_ninv[GQ_MAX_PQBX + 1] = {0.0,      -1.0,      -1.0 / 2,  -1.0 / 3,  -1.0 / 4,  -1.0 / 5,
+                                               -1.0 / 6, -1.0 / 7,  -1.0 / 8,  -1.0 / 9,  -1.0 / 10, -1.0 / 11,
+                                               -1.0 / 12, -1.0 / 13, -1.0 / 14, -1.0 / 15, -1.0 / 16};
+
+// 2^(e - 1023), subnormal and infinite ends included
+__device__ __forceinline__ double pow2_clamped(int e) {
+    return e >= 2047 ? __longlong_as_double(0x7ff0000000000000ll)
+                     : e > 0 ? __longlong_as_double((long long)e << 52)
+                             : e > -52 ? __longlong_as_double(1ll << (51 + e)) : 0.0;
+}
+
+// biased exponent of a strength: 0 for zero only (1 for a subnormal)
+__device__ __forceinline__ int str_expo(double x) {
+    const int e = fx_expo(fx_bits(x));
+    return e > 0 ? e : x != 0.0;
+}
+
+// The lane and slot that hold entry i after a warp_reduce_scatter over n values.
+struct RsPlace {
+    int lane, slot;
+};
+constexpr RsPlace rs_place(int n, int i) {
+    int lane = 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const int h = (n + 1) / 2;
+        if (i >= h) {
+            lane |= o;
+            i -= h;
+        }
+        n = h;
+    }
+    return RsPlace{lane, i};
+}
+
+// The sources [v0, v1) of the loaded ranges in FP64, order by order (every warp
+// lane takes part): any strength or distance, infinities and NaN included.
+template <int KERNEL>
+__device__ __noinline__ void near_centre_slow(const EvalView &E, const NearRanges &R, int v0, int v1, double2 cz, double rc,
+                                              int QQ, int qc, double2 *dst, bool first) {
+    const int lane = threadIdx.x & 31;
+    for (int m = 0; m <= QQ; ++m) {
+        double2 acc = make_double2(0.0, 0.0);
+        int r = 0;
+        if (m <= qc)
+            for (int v = v0 + lane; v < v1; v += 32) {
+                while (R.pre[r + 1] <= v) ++r;
+                const int s = R.beg[r] + (v - R.pre[r]);
+                const double2 y = E.s_xy[s], st = E.str[s];
+                const double wx = y.x - cz.x, wy = y.y - cz.y, n2 = wx * wx + wy * wy;
+                if (KERNEL != GQ_D && m == 0) {
+                    // a coincident source has log term 0
+                    acc.x = fma(st.x, n2 == 0.0 ? 0.0 : gq_log_half(n2, E.logt), acc.x);
+                    continue;
+                }
+                const double inv = gq_rcp(n2);
+                const double2 winv = make_double2(wx * inv, -wy * inv);
+                const double2 u = make_double2(rc * winv.x, rc * winv.y);
+                double2 t = KERNEL == GQ_D ? cmul(st, winv) : make_double2(st.x * u.x, st.x * u.y);
+                for (int i = KERNEL == GQ_D ? 0 : 1; i < m; ++i) t = cmul(t, u);
+                acc = cadd(acc, t);
+            }
+        for (int o = 16; o > 0; o >>= 1)
+            acc = cadd(acc, make_double2(__shfl_xor_sync(0xffffffffu, acc.x, o), __shfl_xor_sync(0xffffffffu, acc.y, o)));
+        if (lane == 0) {
+            if (KERNEL != GQ_D && m >= 1) acc = cscale(acc, c_ninv[m]);
+            dst[m] = first ? acc : cadd(dst[m], acc);
+        }
+    }
+}
+
+// u = (re / w) 2^62 from w, |w|^2 = n2 and the radius' significand (R, 2^61) and
+// biased exponent: re / M2 by fx_rcp, each component's significand shifted into
+// the common format (a right shift for |u| < 2), complemented for a negative w (a
+// unit of 2^-62 off) and multiplied.  The lowest bit of u is set so that no low
+// word is -2^31, which has no negative.
+__device__ __forceinline__ void fx_ratio(double wx, double wy, uint64_t nb, gfx R, int er, gfx &ux, gfx &uy, gfx &nuy) {
+    const gfx G = fx_bal(fx_shl(fx_mul(R, fx_bal(fx_rcp(fx_mant(nb)))), 2));   // 2^61 r / M
+    const int k = er - fx_expo(nb) - 1023 - 1;
+    auto comp = [&](uint64_t b) {
+        const gfx x = fx_bal((long long)fx_shr(fx_mant(b) << 10, -(k + fx_expo(b))) ^ ((long long)b >> 63));
+        return fx_bal(fx_shl(fx_mul(x, G), 4) | 1);
+    };
+    ux = comp(fx_bits(wx));
+    nuy = comp(fx_bits(wy));
+    uy.h = -nuy.h;
+    uy.l = -nuy.l;
+}
+
+// Blocks an SM is compiled for: the sums take 4 (QQ + 1) registers, and the chains
+// of dependent multiply-adds want warps to hide them (q = 8, 1.05 M quadrature
+// nodes: 3 blocks 4.04 ms, 4 3.60, 5 3.39, 7 3.31).
+constexpr int fx_min_blocks(int q) { return q <= 8 ? 7 : q <= 12 ? 5 : 4; }
+template <int QQ, int KERNEL>
+__global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centres_fx(EvalView E, const int *__restrict__ work,
+                                                                   double2 *__restrict__ Qout) {
+    constexpr int NV = 2 * (QQ + 1);
+    typedef typename FxStr<KERNEL>::T str_t;
+    __shared__ NearRanges R;
+    __shared__ int wsum[kFxWarps];
+    __shared__ double2 sy[kFxTile];
+    __shared__ str_t sq[kFxTile];
+    __shared__ long long shl_[KERNEL == GQ_D ? 1 : kFxLogJ];
+    __shared__ int stj[KERNEL == GQ_D ? 1 : kFxLogJ];
+    __shared__ long long ssum[KERNEL == GQ_D ? 1 : 2 * kFxWarps];
+    __shared__ int smax[kFxWarps];
+    if (KERNEL != GQ_D)
+        for (int i = threadIdx.x; i < kFxLogJ; i += kNearThreads) {
+            shl_[i] = E.fxlog->hl[i];
+            stj[i] = E.fxlog->t[i];
+        }
+    const int b = work[blockIdx.x];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ne = (E.loff[0][b + 1] - E.loff[0][b]) + (E.loff[2][b + 1] - E.loff[2][b]) + (E.loff[4][b + 1] - E.loff[4][b]);
+    const int cb = E.ctr_beg[b], ce = E.ctr_end[b];
+    // exponent of the box's rho^2: the logarithms are taken relative to it
+    const double rho = box_rho(E.R, E.blev[b]);
+    const int eref = 2 * fx_expo(fx_bits(rho)) - 1023;
+    bool first = true;
+    for (int e0 = 0; e0 < ne || first; e0 += kNearRanges) {
+        __syncthreads();
+        load_ranges(E, b, e0, ne, R, wsum);
+        const int T = R.pre[R.n];
+        for (int v0 = 0; v0 < T || first; v0 += kFxTile) {
+            const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
+            if (v0) __syncthreads();
+            // the tile's largest strength exponent; strengths are then held as
+            // q 2^(1022 - qe) <= 1/2 (D: each component, so that |d| <= 0.36)
+            int mx = 0;
+            for (int r = w; r < R.n; r += kFxWarps) {
+                const int p0 = R.pre[r], p1 = R.pre[r + 1];
+                for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
+                    const double2 st = E.str[R.beg[r] + (v - p0)];
+                    mx = max(mx, str_expo(st.x));
+                    if (KERNEL == GQ_D) mx = max(mx, str_expo(st.y));
+                }
+            }
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            if (lane == 0) smax[w] = mx;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kFxWarps; ++k) mx = max(mx, smax[k]);
+            if (mx == 0) mx = 1023;   // all zero
+            const int qe = mx + (KERNEL == GQ_D ? 2 : 1);
+            const bool scaled = mx >= 128 && mx <= 1984;
+            // stage the tile: a warp copies one range at a time
+            long long sh = 0, sl = 0;
+            for (int r = w; r < R.n; r += kFxWarps) {
+                const int p0 = R.pre[r], p1 = R.pre[r + 1];
+                for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
+                    const int s = R.beg[r] + (v - p0);
+                    sy[v - v0] = E.s_xy[s];
+                    const double2 st = E.str[s];
+                    if constexpr (KERNEL == GQ_D) {
+                        const gfx30 a = fx_split30(fx_from_double(st.x, qe + 2));
+                        const gfx30 c = fx_split30(fx_from_double(st.y, qe + 2));
+                        sq[v - v0] = make_int4(a.h, a.l, c.h, c.l);
+                    } else {
+                        const gfx a = fx_bal(fx_from_double(st.x, qe));
+                        sq[v - v0] = make_int2(a.h, a.l);
+                        sh += a.h;
+                        sl += a.l;
+                    }
+                }
+            }
+            if (KERNEL != GQ_D) {
+                for (int o = 16; o > 0; o >>= 1) {
+                    sh += __shfl_xor_sync(0xffffffffu, sh, o);
+                    sl += __shfl_xor_sync(0xffffffffu, sl, o);
+                }
+                if (lane == 0) {
+                    ssum[2 * w] = sh;
+                    ssum[2 * w + 1] = sl;
+                }
+            }
+            __syncthreads();
+            for (int c = cb + w; c < ce; c += kFxWarps) {
+                const double2 cz = E.sc_xy[c];
+                const double rc = E.sc_r[c];
+                const int qc = E.qc ? E.qc[c] : QQ;
+                double2 *dst = Qout + (size_t)c * (QQ + 1);
+                double re = rc;
+                bool slow = !scaled;
+                long long acc[NV];   // S: 0 the log sum, 1 unused, then Re, Im of each order; D: Re, Im of each order
+                for (int pass = 0; !slow; ++pass) {
+                    const uint64_t rb = fx_bits(re);
+                    const gfx Rm = fx_bal((long long)(fx_mant(rb) << 9));
+                    const int er = fx_expo(rb);
+#pragma unroll
+                    for (int i = 0; i < NV; ++i) acc[i] = 0;
+                    unsigned nmin = 0xffffffffu, nmax = 0;   // upper words of |w|^2
+                    for (int v = lane; v < n; v += 32) {
+                        const double2 y = sy[v];
+                        const double wx = y.x - cz.x, wy = y.y - cz.y;
+                        const double n2 = fma(wx, wx, wy * wy);
+                        const uint64_t nb = fx_bits(n2);
+                        nmin = min(nmin, (unsigned)(nb >> 32));
+                        nmax = max(nmax, (unsigned)(nb >> 32));
+                        gfx ux, uy, nuy;
+                        fx_ratio(wx, wy, nb, Rm, er, ux, uy, nuy);
+                        const str_t sv = sq[v];
+                        long long tr, ti;
+                        if constexpr (KERNEL == GQ_D) {
+                            fx_cmul30(gfx30{sv.x, sv.y}, gfx30{sv.z, sv.w}, ux, uy, nuy, tr, ti);
+                            acc[0] += tr;
+                            acc[1] += ti;
+                        } else {
+                            const gfx a{sv.x, sv.y};
+                            acc[0] += fx_mul(a, fx_bal(fx_log_half(nb, eref, shl_, stj)));
+                            tr = fx_mul(a, ux);
+                            ti = fx_mul(a, uy);
+                            acc[2] += tr;
+                            acc[3] += ti;
+                        }
+#pragma unroll
+                        for (int m = KERNEL == GQ_D ? 1 : 2; m <= QQ; ++m) {
+                            if (m % 4 == 0 && m > qc) break;
+                            long long xr, xi;
+                            fx_cmul30(fx_split30(tr), fx_split30(ti), ux, uy, nuy, xr, xi);
+                            tr = xr;
+                            ti = xi;
+                            acc[2 * m] += tr;
+                            acc[2 * m + 1] += ti;
+                        }
+                    }
+                    nmin = __reduce_min_sync(0xffffffffu, nmin);
+                    nmax = __reduce_max_sync(0xffffffffu, nmax);
+                    if (n == 0) break;
+                    // |w|^2 a normal number far from the range's ends, the logarithms below 14
+                    const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20);
+                    if (emin < 128 || emax > 1920 || er < 128 || er > 1920 ||
+                        (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40))) {
+                        slow = true;
+                        break;
+                    }
+                    // a source inside the disk: |u|^2 > 1 + 1/32
+                    const double wmin2 = __hiloint2double((int)nmin, 0);
+                    if (pass > 0 || re * re <= wmin2 * (1.0 + 1.0 / 32)) break;
+                    re = sqrt(wmin2);
+                }
+                if (slow) {
+                    near_centre_slow<KERNEL>(E, R, v0, v1, cz, rc, QQ, qc, dst, first);
+                    continue;
+                }
+                // exact sum of the log terms as two words; the others at 2^-60 or as close to
+                // it as the warp's sum allows
+                if (KERNEL != GQ_D) {
+                    acc[1] = acc[0] & ((1 << 27) - 1);
+                    acc[0] >>= 27;
+                }
+                unsigned top = 0;
+#pragma unroll
+                for (int i = KERNEL == GQ_D ? 0 : 2; i < NV; ++i) {
+                    const int h = (int)(acc[i] >> 32);
+                    top |= (unsigned)(h ^ (h >> 31));
+                }
+                // each |acc| < 2^(64 - clz); 32 of them have to stay below 2^63
+                const int sh = max(0, 6 - __clz((int)__reduce_or_sync(0xffffffffu, top)));
+                const long long half = (1ll << sh) >> 1;
+#pragma unroll
+                for (int i = KERNEL == GQ_D ? 0 : 2; i < NV; ++i) acc[i] = (acc[i] + half) >> sh;
+                int base, cnt;
+                warp_reduce_scatter(acc, 0ll, lane, [](long long a, long long x) { return a + x; },
+                                    [](long long x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); }, base, cnt);
+                long long lo = 0;
+                if (KERNEL != GQ_D) {
+                    constexpr RsPlace p1 = rs_place(NV, 1);
+                    lo = __shfl_sync(0xffffffffu, acc[p1.slot], p1.lane);
+                }
+                const double sc = pow2_clamped(qe + 1 - 55), sct = pow2_clamped(qe + 1 - 60 + sh);
+                double *d = reinterpret_cast<double *>(dst);
+#pragma unroll
+                for (int j = 0; j < (NV + 31) / 32; ++j)
+                    if (j < cnt) {
+                        const int i = base + j, m = i >> 1;
+                        double x;
+                        if (KERNEL != GQ_D && m == 0) {
+                            x = 0.0;
+                            if (i == 0) {
+                                long long qh = 0, ql = 0;
+#pragma unroll
+                                for (int k = 0; k < kFxWarps; ++k) {
+                                    qh += ssum[2 * k];
+                                    ql += ssum[2 * k + 1];
+                                }
+                                // sum q (2^62) = qh 2^32 + ql; the log terms have 2^55
+                                const double sumq = fma((double)qh, 4294967296.0, (double)ql);
+                                x = fma((double)acc[0], 134217728.0, (double)lo) * sc +
+                                    sumq * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264);
+                            }
+                        } else {
+                            x = m <= qc ? (double)acc[j] * sct : 0.0;
+                            if (KERNEL != GQ_D) x *= c_ninv[m];
+                            if (re != rc)
+                                for (int k = 0; k < m; ++k) x *= rc / re;
+                            if (KERNEL == GQ_D) x /= re;
+                        }
+                        d[i] = first ? x : d[i] + x;
+                    }
+            }
+            first = false;
+        }
+    }
+}
+
+template <int QQ>
+void launch_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Q) {
+    auto kd = k_near_centres_fx<QQ, GQ_D>;
+    auto ks = k_near_centres_fx<QQ, GQ_S>;
+    GQ_LAUNCH(ctx, (E.kernel == GQ_D ? kd : ks), nwork, kNearThreads, 0, E, work, Q);
+}
+
+}  // namespace
+
+void gq_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Q) {
+    switch (E.Q) {
+#define GQ_CASE(v) case v: launch_near_centres_fx<v>(ctx, E, nwork, work, Q); break;
+        GQ_CASE(1) GQ_CASE(2) GQ_CASE(3) GQ_CASE(4) GQ_CASE(5) GQ_CASE(6) GQ_CASE(7) GQ_CASE(8)
+        GQ_CASE(9) GQ_CASE(10) GQ_CASE(11) GQ_CASE(12) GQ_CASE(13) GQ_CASE(14) GQ_CASE(15) GQ_CASE(16)
+#undef GQ_CASE
+        default: throw gq_error{GQ_ERR_INVALID, "p_qbx out of range"};
+    }
+}

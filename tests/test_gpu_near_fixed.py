@@ -1,0 +1,135 @@
+"""Direct sums to the QBX centres in fixed point (k_near_centres_fx) against
+direct sums in long double: one box holds everything (n_max above the particle
+count), so the QBX coefficients are the kernel's alone.
+
+The tolerance is FP64's own for these sums: each term is a product of at most
+q + 4 rounded factors and each sum has n terms, (q + 4 + log2 n) 2^-53 of the
+absolute sum at worst; the fixed-point terms and sums are rounded below that of
+the largest term, which the nearest source's |u| ~ 1 makes part of the sum."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+
+def _geo(g, q):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_04070_gb300 import Geometry, params_default
+    geo = Geometry(g, params_default(p_qbx=q, p_fmm=10, n_max=100000))
+    geo.build()
+    assert geo.nbox == 1
+    return geo
+
+
+def _problem(panels, nu=64, seed=5):
+    g = workloads.starfish.discretize([workloads.Curve(modes=((3, 0.25, 0.3),))], panels, nu=nu)
+    rng = np.random.default_rng(seed)
+    g["density"] = rng.normal(size=len(g["base_xy"]))
+    g["tgt_xy"] = g["base_xy"]
+    g["tgt_onsurf"] = np.arange(len(g["base_xy"]), dtype=np.int32)
+    return g
+
+
+def _strengths(g, mu):
+    rb, ru = g["ref_b"], g["ref_u"]
+    L = np.array([[np.prod([(x - rb[k]) / (rb[j] - rb[k]) for k in range(len(rb)) if k != j]) for j in range(len(rb))]
+                  for x in ru])
+    return (mu.reshape(-1, len(rb)) @ L.T).ravel() * g["up_w"]
+
+
+def _reference(g, kern, q, mu, sel, c, r):
+    """Coefficients of the centres `sel` and, per order, the absolute sums."""
+    f = np.longdouble
+    qs = _strengths(g, mu).astype(f)
+    st = qs * (g["up_n"][:, 0].astype(f) + 1j * g["up_n"][:, 1].astype(f)) if kern == "D" else qs + 0j
+    y = g["up_xy"][:, 0].astype(f) + 1j * g["up_xy"][:, 1].astype(f)
+    w = y[None, :] - (c[sel, 0].astype(f) + 1j * c[sel, 1].astype(f))[:, None]
+    u = r[sel].astype(f)[:, None] / w
+    out, mag = [], []
+    for m in range(q + 1):
+        if kern == "D":
+            t = st / w * u ** m
+        elif m == 0:
+            t = qs * np.log(np.abs(w)) + 0j
+        else:
+            t = -st * u ** m / f(m)
+        out.append(t.sum(1))
+        mag.append(np.abs(t).sum(1))
+    return np.stack(out, 1), np.stack(mag, 1)
+
+
+def _check(g, kern, q, mu=None, sel=None):
+    geo = _geo(g, q)
+    mu = g["density"] if mu is None else mu
+    c, r, _ = geo.centres()
+    sel = np.arange(0, len(r), 7) if sel is None else sel
+    geo.eval(kern, mu)
+    got = geo.qbx_coefficients()[sel] * r[sel, None] ** np.arange(q + 1)
+    ref, mag = _reference(g, kern, q, mu, sel, c, r)
+    if kern == "S":
+        got[:, 0], ref[:, 0] = got[:, 0].real, ref[:, 0].real
+    # + 4: the scaling by r^m and its inverse in the export and here
+    tol = (q + 8 + np.log2(len(g["up_w"]))) * 2.0 ** -53 * np.maximum(mag, np.abs(_strengths(g, mu)).max())
+    assert (np.abs(got - ref) <= tol).all(), (np.abs(got - ref) / tol).max()
+    geo.close()
+
+
+# tiles of 384 sources: below, at and above one and two of them; a warp's 32 lanes not filled
+@pytest.mark.parametrize("kern", ["S", "D"])
+@pytest.mark.parametrize("panels,nu,q", [(8, 17, 5), (8, 47, 1), (8, 48, 8), (11, 35, 8), (12, 64, 3), (13, 60, 16), (24, 64, 8)])
+def test_tile_edges(kern, panels, nu, q):
+    _check(_problem(panels, nu), kern, q)
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+@pytest.mark.parametrize("dist", [0.97, 0.5, 0.01, 1e-7])
+def test_source_inside_the_disk(kern, dist):
+    """A source at dist r from a centre: its centre is summed again with the
+    distance as radius (1e-7: FP64 order by order for S)."""
+    g = _problem(16)
+    geo = _geo(g, 8)
+    c, r, _ = geo.centres()
+    geo.close()
+    g["up_xy"] = g["up_xy"].copy()
+    g["up_xy"][100] = c[50] + dist * r[50] * np.array([0.6, 0.8])
+    _check(g, kern, 8, sel=np.array([50, 51, 200]))
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+def test_strength_ranges(kern):
+    g = _problem(16)
+    mu = g["density"]
+    _check(g, kern, 5, mu=np.ldexp(mu, 400))
+    _check(g, kern, 5, mu=np.ldexp(mu, -400))
+    weak = mu.copy()
+    weak[64:] *= 2.0 ** -30
+    _check(g, kern, 5, mu=weak)
+    geo = _geo(g, 5)
+    assert (geo.eval(kern, np.zeros_like(mu)) == 0).all()
+    bad = mu.copy()
+    bad[3] = np.inf
+    assert np.isnan(geo.eval(kern, bad)).all()
+    tiny = geo.eval(kern, np.ldexp(mu, -1000))   # outside the scaled range: FP64 sums
+    base = geo.eval(kern, mu)
+    assert np.abs(np.ldexp(tiny, 1000) - base).max() <= 1e-13 * np.abs(base).max()
+    geo.close()
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+def test_source_at_a_centre(kern):
+    """|w| = 0: NaN for the targets of that centre, the others unharmed."""
+    g = _problem(16)
+    geo = _geo(g, 5)
+    c, r, _ = geo.centres()
+    geo.close()
+    g["up_xy"] = g["up_xy"].copy()
+    g["up_xy"][100] = c[50]
+    geo = _geo(g, 5)
+    v = geo.eval(kern, g["density"])
+    geo.close()
+    assert np.isnan(v[25]) and np.isfinite(np.delete(v, 25)).all()
+    _check(g, kern, 5, sel=np.array([10, 51, 200]))
