@@ -125,3 +125,6 @@ __device__ __forceinline__ void warp_reduce_scatter(V (&v)[NV], V zero, int lane
 
 // direct sums to the QBX centres in 64-bit fixed point (gq_near_fx.cu): Qout [nc][E.Q+1]
 void gq_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Qout);
+// List 2 translations (M2L) of orders 16 .. 30 in fixed point (gq_m2l_fx.cu), added to L
+void gq_m2l_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *L);
+void gq_m2l_fx_prepare(int dev);   // its tables on device dev

@@ -1896,6 +1896,7 @@ static const ConstTables &const_tables(int dev) {
     gq_log_table_host(&LT);
     GqDflLogTable DT;
     gq_dfl_log_table_host(&DT);
+    gq_m2l_fx_prepare(dev);
     ConstTables C;
     C.logt = upload_const((const double *)&LT, kGqLogN);
     FxLogTable FT;
@@ -2185,8 +2186,8 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                   (const double2 *)g->M, g->M2.p);
     // Stage 4
     if (g->n_far_boxes) {
-        int G = P1 <= 16 ? 16 : 32;
         if (m2l_split) {
+            const int G = P1 <= 16 ? 16 : 32;
             size_t sm = sizeof(float2) * P1 * (P1 | 1);
             auto k16 = k_m2l_split<16>;
             auto k32 = k_m2l_split<32>;
@@ -2194,11 +2195,11 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                       g->n_far_boxes, (const int *)g->far_boxes, T.dtab2, T.logtab2, T.binom2, g->L2.p);
         } else if (gq_m2l_tc_supported(g)) {
             gq_m2l_tc(g, (const double2 *)g->M, g->L.p);   // FP64-accurate, on the tensor cores
+        } else if (P1 > 16) {
+            gq_m2l_fx(g, E, (const double2 *)g->M, g->L.p);   // in fixed point
         } else {
-            size_t sm = sizeof(double) * P1 * P1;
             auto k16 = k_m2l<16>;
-            auto k32 = k_m2l<32>;
-            GQ_LAUNCH(ctx, (G == 16 ? k16 : k32), gq_blocks((long long)g->n_far_boxes * G, 128), 128, sm, E,
+            GQ_LAUNCH(ctx, k16, gq_blocks((long long)g->n_far_boxes * 16, 128), 128, sizeof(double) * P1 * P1, E,
                       g->n_far_boxes, (const int *)g->far_boxes, (const double2 *)g->M, (const double2 *)T.dtab,
                       (const double *)T.logtab, g->L.p);
         }

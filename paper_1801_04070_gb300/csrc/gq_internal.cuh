@@ -151,6 +151,8 @@ struct gq_geom {
     dbuf<double2> strength;          // sorted sources: S -> (q, 0), D -> d
     dbuf<unsigned int> qexp;         // largest biased exponent of the strengths (one value)
     dbuf<double2> M, L;              // [nbox][p_fmm+1] box-scaled expansions
+    dbuf<int4> Mfx;                  // [nbox][p_fmm+1] multipoles in fixed point (gq_m2l_fx.cu)
+    dbuf<int> Efx;                   // [nbox] their exponents
     dbuf<double2> Q;                 // [nc][p_qbx+1] r-scaled QBX coefficients (sorted centres): far part
     dbuf<double2> Qn;                // the same, direct part
     dbuf<double> pot;                // sorted point targets: Re Phi, far part

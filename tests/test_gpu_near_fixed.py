@@ -133,3 +133,31 @@ def test_source_at_a_centre(kern):
     geo.close()
     assert np.isnan(v[25]) and np.isfinite(np.delete(v, 25)).all()
     _check(g, kern, 5, sel=np.array([10, 51, 200]))
+
+
+@pytest.mark.parametrize("p", [16, 17, 23, 30])
+def test_list2_in_fixed_point(p):
+    """List 2 of the orders 16 .. 30 (k_m2l_fx) against the FP64 kernels of the
+    no-allocation evaluation, on a tree with several levels of List 2 entries
+    and odd list lengths.  Both round the far field at 2^-53 of its largest
+    terms; 1e-13 is the bound the other List 2 comparisons use."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import ctypes as C
+
+    from paper_1801_04070_gb300 import Geometry, params_default
+    from paper_1801_04070_gb300 import _lib
+    g = workloads.small_grid(3, 2, 24, 2000, seed=p)
+    geo = Geometry(g, params_default(p_qbx=5, p_fmm=p, n_max=32))
+    geo.build()
+    assert geo.info.list_size[1] > 1000
+    dens = torch.tensor(g["density"], dtype=torch.float64, device="cuda")
+    for kern in ("S", "D"):
+        a = torch.empty(geo.nt, dtype=torch.float64, device="cuda")
+        b = torch.empty_like(a)
+        geo.eval(kern, dens, a)
+        geo._check(geo.L.gq_eval_noalloc(geo._geom, _lib.KERNELS[kern], C.c_void_p(dens.data_ptr()), C.c_void_p(b.data_ptr())))
+        torch.cuda.synchronize()
+        assert (a - b).abs().max().item() <= 1e-13 * b.abs().max().item(), kern
+    geo.close()
