@@ -32,13 +32,7 @@ __host__ __device__ constexpr int woff(int l) {
     return l == 0 ? 0 : woff(l - 1) + (l == 1 ? 32 * 64 + 64 : l == 2 ? 64 * 32 + 32 : l == 3 ? 32 * 32 + 32 : 32 * 2 + 2);
 }
 constexpr int kNParams = woff(kLayers);
-// the same layout for device code (runtime layer index)
-__device__ __forceinline__ int ddim(int l) { return l == 0 ? 32 : l == 1 ? 64 : l == 2 ? 32 : l == 3 ? 32 : 2; }
-__device__ __forceinline__ int dwoff(int l) {
-    int o = 0;
-    for (int i = 0; i < l; ++i) o += ddim(i) * ddim(i + 1) + ddim(i + 1);
-    return o;
-}
+__host__ __device__ constexpr int cdim(int l) { return l == 1 ? 64 : l == 4 ? 2 : 32; }   // kDims, for device code
 
 // ------------------------------------------------------------------ features
 // curvature at base nodes from the turning of the normal between the
@@ -118,76 +112,229 @@ __global__ void k_centre_features(int nc, int nb, int nu, const int *__restrict_
 }
 
 // ------------------------------------------------------------------ MLP kernels
-// Z = A_prev W^T + b, A = relu(Z) (or A = Z for the last layer); thread per (sample, neuron)
-__global__ void k_dense_fwd(int B, int nin, int nout, const float *__restrict__ Ain, const float *__restrict__ W,
-                            const float *__restrict__ bias, float *__restrict__ Z, float *__restrict__ A, int relu) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B * nout) return;
-    int s = t / nout, o = t % nout;
-    const float *a = Ain + (size_t)s * nin, *w = W + (size_t)o * nin;
-    float z = bias[o];
-    for (int i = 0; i < nin; ++i) z = fmaf(w[i], a[i], z);
-    Z[t] = z;
-    A[t] = relu ? fmaxf(z, 0.f) : z;
+// A training step is two launches: k_mlp_samples (gather, forward, error,
+// deltas; samples are independent) and k_mlp_params (gradient and Adam;
+// parameters are independent).  One launch per layer and pass (13 a step, each
+// thread reading its operands from L2) took 0.35 ms a step of 1,024 samples;
+// these two about 0.015 ms.  Every sum keeps its order (over inputs, outputs or
+// samples, ascending, from the same start), so the trained weights are
+// unchanged bit for bit.
+constexpr int kSB = 8;            // samples per block of k_mlp_samples
+constexpr int kPT = 128;          // weights per block of k_mlp_params
+constexpr int kChunk = 64;        // samples staged at a time by k_mlp_params
+
+// activations and deltas of a batch, per layer [B][width]
+struct MlpBatch {
+    float *X;                     // inputs as used (normalised when training)
+    float *A[kLayers];            // layer outputs
+    float *D[kLayers];            // d loss / d (layer output before ReLU)
+    double *sse;                  // per block of k_mlp_samples: sum of squared errors (may be null)
+};
+
+template <int L>
+__device__ __forceinline__ void mlp_forward(const float *sw, const float *in, float *out, int nb, int s0, float *gout) {
+    constexpr int NI = cdim(L), NO = cdim(L + 1), LD = NI + 1;
+    for (int t = threadIdx.x; t < kSB * NO; t += blockDim.x) {
+        const int s = t / NO, o = t % NO;
+        const float *a = in + s * NI, *w = sw + o * LD;
+        float z = sw[NO * LD + o];
+#pragma unroll 16
+        for (int i = 0; i < NI; ++i) z = fmaf(w[i], a[i], z);
+        if (L < kLayers - 1) z = fmaxf(z, 0.f);
+        out[t] = z;
+        if (s < nb) gout[(size_t)(s0 + s) * NO + o] = z;
+    }
+    __syncthreads();
 }
 
-// delta = 2 (Yhat - Y) / (B * nout); per-sample squared error into err
-__global__ void k_mse_delta(int B, int nout, const float *__restrict__ Yh, const float *__restrict__ Y,
-                            float *__restrict__ delta, float *__restrict__ err) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B * nout) return;
-    float d = Yh[t] - Y[t];
-    delta[t] = 2.f * d / (float)(B * nout);
-    err[t] = d * d;
+// delta_prev = (W^T delta) relu', relu' = 1 where the layer's output is positive
+template <int L>
+__device__ __forceinline__ void mlp_backward(const float *sw, const float *delta, const float *aprev, float *dprev, int nb,
+                                             int s0, float *gout) {
+    constexpr int NI = cdim(L), NO = cdim(L + 1), LD = NI + 1;
+    for (int t = threadIdx.x; t < kSB * NI; t += blockDim.x) {
+        const int s = t / NI, i = t % NI;
+        float g = 0.f;
+#pragma unroll 16
+        for (int o = 0; o < NO; ++o) g = fmaf(delta[s * NO + o], sw[o * LD + i], g);
+        g = aprev[t] > 0.f ? g : 0.f;
+        dprev[t] = g;
+        if (s < nb) gout[(size_t)(s0 + s) * NI + i] = g;
+    }
+    __syncthreads();
 }
 
-// dW[o][i] = sum_s delta[s][o] A[s][i], db[o] = sum_s delta[s][o]; thread per parameter
-__global__ void k_dense_grad(int B, int nin, int nout, const float *__restrict__ delta, const float *__restrict__ Ain,
-                             float *__restrict__ dW, float *__restrict__ db) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nout * (nin + 1)) return;
-    if (t < nout * nin) {
-        int o = t / nin, i = t % nin;
-        float g = 0.f;
-        for (int s = 0; s < B; ++s) g = fmaf(delta[(size_t)s * nout + o], Ain[(size_t)s * nin + i], g);
-        dW[t] = g;
-    } else {
-        int o = t - nout * nin;
-        float g = 0.f;
-        for (int s = 0; s < B; ++s) g += delta[(size_t)s * nout + o];
-        db[o] = g;
+// offset of layer l's weights in shared memory (rows padded by one word)
+__host__ __device__ constexpr int swoff(int l) {
+    return l == 0 ? 0 : swoff(l - 1) + cdim(l) * (cdim(l - 1) + 1) + cdim(l);
+}
+
+// Rows perm[s] (or row s) of X and Y, standardised when mu and sd are given.
+__global__ void __launch_bounds__(256) k_mlp_samples(int B, const int *__restrict__ perm, const float *__restrict__ X,
+                                                     const float *__restrict__ Y, const float *__restrict__ xmu,
+                                                     const float *__restrict__ xsd, const float *__restrict__ ymu,
+                                                     const float *__restrict__ ysd, const float *__restrict__ w, MlpBatch M) {
+    __shared__ float sw[swoff(kLayers)];
+    __shared__ float x[kSB * 32], a0[kSB * 64], a1[kSB * 32], a2[kSB * 32], a3[kSB * 2], d3[kSB * 2], da[kSB * 64], db[kSB * 64];
+    __shared__ float se[kSB * 2];
+    const int s0 = blockIdx.x * kSB, nb = min(kSB, B - s0);
+#pragma unroll
+    for (int l = 0; l < kLayers; ++l) {
+        const int ni = cdim(l), no = cdim(l + 1);
+        for (int t = threadIdx.x; t < no * ni; t += blockDim.x) sw[swoff(l) + t / ni * (ni + 1) + t % ni] = w[woff(l) + t];
+        for (int t = threadIdx.x; t < no; t += blockDim.x) sw[swoff(l) + no * (ni + 1) + t] = w[woff(l) + no * ni + t];
+    }
+    for (int t = threadIdx.x; t < kSB * kNF; t += blockDim.x) {
+        const int s = t / kNF, c = t % kNF;
+        float v = 0.f;
+        if (s < nb) {
+            v = X[(size_t)(perm ? perm[s0 + s] : s0 + s) * kNF + c];
+            if (xmu) v = (v - xmu[c]) / xsd[c];
+            M.X[(size_t)(s0 + s) * kNF + c] = v;
+        }
+        x[t] = v;
+    }
+    __syncthreads();
+    mlp_forward<0>(sw + swoff(0), x, a0, nb, s0, M.A[0]);
+    mlp_forward<1>(sw + swoff(1), a0, a1, nb, s0, M.A[1]);
+    mlp_forward<2>(sw + swoff(2), a1, a2, nb, s0, M.A[2]);
+    mlp_forward<3>(sw + swoff(3), a2, a3, nb, s0, M.A[3]);
+    // delta = 2 (Yhat - Y) / (2 B)
+    if (threadIdx.x < kSB * 2) {
+        const int t = threadIdx.x, s = t / 2, c = t % 2;
+        float d = 0.f;
+        if (s < nb) {
+            float y = Y[(size_t)(perm ? perm[s0 + s] : s0 + s) * 2 + c];
+            if (ymu) y = (y - ymu[c]) / ysd[c];
+            d = a3[t] - y;
+            M.D[3][(size_t)(s0 + s) * 2 + c] = 2.f * d / (float)(B * 2);
+        }
+        d3[t] = 2.f * d / (float)(B * 2);
+        se[t] = d * d;
+    }
+    __syncthreads();
+    if (M.sse && threadIdx.x == 0) {
+        double e = 0.0;
+        for (int t = 0; t < kSB * 2; ++t) e += se[t];
+        M.sse[blockIdx.x] = e;
+    }
+    mlp_backward<3>(sw + swoff(3), d3, a2, da, nb, s0, M.D[2]);
+    mlp_backward<2>(sw + swoff(2), da, a1, db, nb, s0, M.D[1]);
+    mlp_backward<1>(sw + swoff(1), db, a0, da, nb, s0, M.D[0]);
+}
+
+struct AdamStep {
+    float *w, *m, *v;             // null w: gradient only
+    float lr, b1, b2, c1, c2;
+};
+
+// Gradient of kPT weights of layer L (whole output rows) and of their rows'
+// biases, summed over the samples in order; the samples' activations and deltas
+// come through shared memory, a chunk ahead of the sums.
+template <int L>
+__device__ __forceinline__ void mlp_params_layer(int blk, int B, const MlpBatch &M, float *__restrict__ grad,
+                                                 const AdamStep &ad, float (*sA)[kChunk * 64], float (*sD)[kChunk * 4]) {
+    constexpr int NI = cdim(L), NO = cdim(L + 1), R = kPT / NI < NO ? kPT / NI : NO;
+    const float *Ain = L == 0 ? M.X : M.A[L > 0 ? L - 1 : 0], *D = M.D[L];
+    const int o0 = blk * R, tid = threadIdx.x;
+    auto stage = [&](int s0, int buf) {
+        const int n = min(kChunk, B - s0);
+        for (int t = tid; t < n * NI / 4; t += blockDim.x) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(&sA[buf][t * 4]);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(Ain + (size_t)s0 * NI + t * 4));
+        }
+        for (int t = tid; t < n * R; t += blockDim.x) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(&sD[buf][t]);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(D + (size_t)(s0 + t / R) * NO + o0 + t % R));
+        }
+        asm volatile("cp.async.commit_group;");
+    };
+    // thread: a weight (r, i), or a bias of row r
+    const bool isw = tid < R * NI, isb = tid >= kPT && tid < kPT + R;
+    const int r = isw ? tid / NI : tid - kPT, i = tid % NI;
+    float g = 0.f;
+    stage(0, 0);
+    for (int s0 = 0, buf = 0; s0 < B; s0 += kChunk, buf ^= 1) {
+        if (s0 + kChunk < B) {
+            stage(s0 + kChunk, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;");
+        } else {
+            asm volatile("cp.async.wait_group 0;");
+        }
+        __syncthreads();
+        const int n = min(kChunk, B - s0);
+        if (isw) {
+#pragma unroll 16
+            for (int s = 0; s < n; ++s) g = fmaf(sD[buf][s * R + r], sA[buf][s * NI + i], g);
+        } else if (isb) {
+#pragma unroll 16
+            for (int s = 0; s < n; ++s) g += sD[buf][s * R + r];
+        }
+        __syncthreads();
+    }
+    if (!isw && !isb) return;
+    const int p = woff(L) + (isw ? (o0 + r) * NI + i : NO * NI + o0 + r);
+    grad[p] = g;
+    if (ad.w) {
+        const float mi = ad.b1 * ad.m[p] + (1.f - ad.b1) * g, vi = ad.b2 * ad.v[p] + (1.f - ad.b2) * g * g;
+        ad.m[p] = mi;
+        ad.v[p] = vi;
+        ad.w[p] -= ad.lr * (mi / ad.c1) / (sqrtf(vi / ad.c2) + 1e-8f);
     }
 }
 
-// delta_prev[s][i] = (sum_o delta[s][o] W[o][i]) * relu'(Z_prev[s][i])
-__global__ void k_dense_bwd(int B, int nin, int nout, const float *__restrict__ delta, const float *__restrict__ W,
-                            const float *__restrict__ Zprev, float *__restrict__ dprev) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B * nin) return;
-    int s = t / nin, i = t % nin;
-    float g = 0.f;
-    for (int o = 0; o < nout; ++o) g = fmaf(delta[(size_t)s * nout + o], W[(size_t)o * nin + i], g);
-    dprev[t] = Zprev[t] > 0.f ? g : 0.f;
+__host__ __device__ constexpr int mlp_param_blocks(int l) { return (cdim(l) * cdim(l + 1) + kPT - 1) / kPT; }
+
+__global__ void __launch_bounds__(kPT + 32) k_mlp_params(int B, MlpBatch M, float *__restrict__ grad, AdamStep ad) {
+    __shared__ __align__(16) float sA[2][kChunk * 64];
+    __shared__ float sD[2][kChunk * 4];
+    constexpr int b1 = mlp_param_blocks(0), b2 = b1 + mlp_param_blocks(1), b3 = b2 + mlp_param_blocks(2);
+    const int b = blockIdx.x;
+    if (b < b1) mlp_params_layer<0>(b, B, M, grad, ad, sA, sD);
+    else if (b < b2) mlp_params_layer<1>(b - b1, B, M, grad, ad, sA, sD);
+    else if (b < b3) mlp_params_layer<2>(b - b2, B, M, grad, ad, sA, sD);
+    else mlp_params_layer<3>(b - b3, B, M, grad, ad, sA, sD);
 }
 
-__global__ void k_adam(int n, float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, float lr, float b1, float b2, float c1, float c2) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float gi = g[i];
-    float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+// Column sums and sums of squares of X [n][d] (d = 32 or 2) in FP64: per block
+// part[block][2 d], then k_col_stats makes mean and deviation (1 where it is
+// below 1e-6) of the blocks' parts, in order.
+constexpr int kStatBlocks = 64;
+__global__ void __launch_bounds__(256) k_col_sums(int n, int d, const float *__restrict__ X, double *__restrict__ part) {
+    __shared__ double s1[256], s2[256];
+    const int c = threadIdx.x % d, rows = blockDim.x / d;
+    double a = 0.0, b = 0.0;
+    for (int i = blockIdx.x * rows + threadIdx.x / d; i < n; i += gridDim.x * rows) {
+        const double x = X[(size_t)i * d + c];
+        a += x;
+        b += x * x;
+    }
+    s1[threadIdx.x] = a;
+    s2[threadIdx.x] = b;
+    __syncthreads();
+    if (threadIdx.x < d) {
+        for (int r = 1; r < rows; ++r) {
+            a += s1[r * d + c];
+            b += s2[r * d + c];
+        }
+        part[(size_t)blockIdx.x * 2 * d + c] = a;
+        part[(size_t)blockIdx.x * 2 * d + d + c] = b;
+    }
 }
 
-// rows perm[k] of X (n x d) into out (B x d), normalised (x - mu) / sd
-__global__ void k_gather_rows(int B, int d, const int *__restrict__ perm, const float *__restrict__ X,
-                              const float *__restrict__ mu, const float *__restrict__ sd, float *__restrict__ out) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= B * d) return;
-    int s = t / d, c = t % d;
-    out[t] = (X[(size_t)perm[s] * d + c] - mu[c]) / sd[c];
+__global__ void k_col_stats(int n, int d, const double *__restrict__ part, float *__restrict__ mu, float *__restrict__ sd) {
+    const int c = threadIdx.x;
+    if (c >= d) return;
+    double s = 0.0, q = 0.0;
+    for (int b = 0; b < kStatBlocks; ++b) {
+        s += part[(size_t)b * 2 * d + c];
+        q += part[(size_t)b * 2 * d + d + c];
+    }
+    const double m = s / n;
+    double v = sqrt(fmax(q / n - m * m, 0.0));
+    if (v < 1e-6) v = 1.0;
+    mu[c] = (float)m;
+    sd[c] = (float)v;
 }
 
 // BF16 inference on the tensor cores (mma.sync m16n8k16, BF16 inputs, FP32
@@ -345,8 +492,7 @@ struct gq_mlp {
     int adam_t = 0;
     // work buffers for a batch
     int cap = 0;
-    dbuf<float> Xb, Yb, Z[kLayers], A[kLayers], D[kLayers], err;
-    dbuf<int> perm;
+    dbuf<float> Xb, A[kLayers], D[kLayers];
 };
 
 namespace {
@@ -354,47 +500,40 @@ namespace {
 void ensure_batch(gq_mlp *M, int B) {
     if (B <= M->cap) return;
     M->Xb.alloc((size_t)B * kNF);
-    M->Yb.alloc((size_t)B * 2);
-    M->err.alloc((size_t)B * 2);
     for (int l = 0; l < kLayers; ++l) {
-        M->Z[l].alloc((size_t)B * kDims[l + 1]);
         M->A[l].alloc((size_t)B * kDims[l + 1]);
         M->D[l].alloc((size_t)B * kDims[l + 1]);
     }
-    M->perm.alloc(B);
     M->cap = B;
 }
 
-// forward + backward on the batch in Xb / Yb (already normalised); gradient into M->g; returns sum of squares
-void fwd_bwd(gq_mlp *M, int B, bool want_err, double *sse) {
-    gq_ctx *ctx = M->ctx;
-    const float *in = M->Xb.p;
+// One batch: forward and backward on rows perm[0 .. B) (or the first B rows) of
+// X and Y, standardised with the network's statistics when norm; the gradient
+// goes to M->g, and with ad.w the Adam step is taken.  sse (may be null): one
+// sum of squared errors per kSB samples.
+void mlp_batch(gq_mlp *M, int B, const int *perm, const float *X, const float *Y, bool norm, double *sse, const AdamStep &ad) {
+    MlpBatch b;
+    b.X = M->Xb;
     for (int l = 0; l < kLayers; ++l) {
-        int nin = kDims[l], nout = kDims[l + 1];
-        GQ_LAUNCH(ctx, k_dense_fwd, gq_blocks((long long)B * nout, kT), kT, 0, B, nin, nout, in,
-                  (const float *)M->w.p + woff(l), (const float *)M->w.p + woff(l) + nin * nout, M->Z[l].p, M->A[l].p,
-                  l < kLayers - 1 ? 1 : 0);
-        in = M->A[l].p;
+        b.A[l] = M->A[l];
+        b.D[l] = M->D[l];
     }
-    GQ_LAUNCH(ctx, k_mse_delta, gq_blocks((long long)B * 2, kT), kT, 0, B, 2, (const float *)M->A[kLayers - 1].p,
-              (const float *)M->Yb.p, M->D[kLayers - 1].p, M->err.p);
-    for (int l = kLayers - 1; l >= 0; --l) {
-        int nin = kDims[l], nout = kDims[l + 1];
-        const float *Ain = l == 0 ? (const float *)M->Xb.p : (const float *)M->A[l - 1].p;
-        GQ_LAUNCH(ctx, k_dense_grad, gq_blocks((long long)nout * (nin + 1), kT), kT, 0, B, nin, nout,
-                  (const float *)M->D[l].p, Ain, M->g.p + woff(l), M->g.p + woff(l) + nin * nout);
-        if (l > 0)
-            GQ_LAUNCH(ctx, k_dense_bwd, gq_blocks((long long)B * nin, kT), kT, 0, B, nin, nout, (const float *)M->D[l].p,
-                      (const float *)M->w.p + woff(l), (const float *)M->Z[l - 1].p, M->D[l - 1].p);
-    }
-    if (want_err) {
-        std::vector<float> e((size_t)B * 2);
-        GQ_CUDA(cudaMemcpyAsync(e.data(), M->err.p, sizeof(float) * e.size(), cudaMemcpyDeviceToHost, ctx->stream));
-        GQ_CUDA(cudaStreamSynchronize(ctx->stream));
-        double s = 0;
-        for (float x : e) s += x;
-        *sse = s;
-    }
+    b.sse = sse;
+    const float *null = nullptr;
+    GQ_LAUNCH(M->ctx, k_mlp_samples, gq_blocks(B, kSB), 256, 0, B, perm, X, Y, norm ? (const float *)M->xmu : null,
+              norm ? (const float *)M->xsd : null, norm ? (const float *)M->ymu : null, norm ? (const float *)M->ysd : null,
+              (const float *)M->w, b);
+    constexpr int blocks = mlp_param_blocks(0) + mlp_param_blocks(1) + mlp_param_blocks(2) + mlp_param_blocks(3);
+    GQ_LAUNCH(M->ctx, k_mlp_params, blocks, kPT + 32, 0, B, b, M->g.p, ad);
+}
+
+double sum_on_host(gq_ctx *ctx, const double *dev, size_t n) {
+    std::vector<double> h(n);
+    GQ_CUDA(cudaMemcpyAsync(h.data(), dev, sizeof(double) * n, cudaMemcpyDeviceToHost, ctx->stream));
+    GQ_CUDA(cudaStreamSynchronize(ctx->stream));
+    double s = 0;
+    for (double x : h) s += x;
+    return s;
 }
 
 const float *to_device(gq_ctx *ctx, const float *p, size_t n, dbuf<float> &tmp, bool is_dev) {
@@ -450,11 +589,11 @@ void gq_mlp_loss_grad_impl(gq_mlp *M, const float *X, const float *Y, int n, boo
     ensure_batch(M, n);
     dbuf<float> tx, ty;
     const float *Xd = to_device(M->ctx, X, (size_t)n * kNF, tx, dev), *Yd = to_device(M->ctx, Y, (size_t)n * 2, ty, dev);
-    GQ_CUDA(cudaMemcpyAsync(M->Xb.p, Xd, sizeof(float) * n * kNF, cudaMemcpyDeviceToDevice, M->ctx->stream));
-    GQ_CUDA(cudaMemcpyAsync(M->Yb.p, Yd, sizeof(float) * n * 2, cudaMemcpyDeviceToDevice, M->ctx->stream));
-    double sse = 0;
-    fwd_bwd(M, n, true, &sse);
-    if (loss) *loss = (float)(sse / (2.0 * n));
+    dbuf<double> sse;
+    sse.alloc(gq_blocks(n, kSB));
+    mlp_batch(M, n, nullptr, Xd, Yd, false, sse.p, AdamStep{});
+    const double e = sum_on_host(M->ctx, sse.p, gq_blocks(n, kSB));
+    if (loss) *loss = (float)(e / (2.0 * n));
     if (grad) GQ_CUDA(cudaMemcpy(grad, M->g.p, sizeof(float) * kNParams, cudaMemcpyDeviceToHost));
 }
 
@@ -467,53 +606,36 @@ double gq_mlp_train_impl(gq_mlp *M, const float *X, const float *Y, int n, bool 
     ensure_batch(M, B);
     dbuf<float> tx, ty;
     const float *Xd = to_device(ctx, X, (size_t)n * kNF, tx, dev), *Yd = to_device(ctx, Y, (size_t)n * 2, ty, dev);
-    // normalisation statistics (host, FP64)
-    std::vector<float> hx((size_t)n * kNF), hy((size_t)n * 2);
-    GQ_CUDA(cudaMemcpyAsync(hx.data(), Xd, sizeof(float) * hx.size(), cudaMemcpyDeviceToHost, st));
-    GQ_CUDA(cudaMemcpyAsync(hy.data(), Yd, sizeof(float) * hy.size(), cudaMemcpyDeviceToHost, st));
-    GQ_CUDA(cudaStreamSynchronize(st));
-    std::vector<float> xmu(kNF), xsd(kNF), ymu(2), ysd(2);
-    for (int c = 0; c < kNF + 2; ++c) {
-        const std::vector<float> &h = c < kNF ? hx : hy;
-        int d = c < kNF ? kNF : 2, cc = c < kNF ? c : c - kNF;
-        double s = 0, s2 = 0;
-        for (int i = 0; i < n; ++i) { double x = h[(size_t)i * d + cc]; s += x; s2 += x * x; }
-        double mu = s / n, sd = sqrt(fmax(s2 / n - mu * mu, 0.0));
-        if (sd < 1e-6) sd = 1.0;
-        (c < kNF ? xmu[cc] : ymu[cc]) = (float)mu;
-        (c < kNF ? xsd[cc] : ysd[cc]) = (float)sd;
+    // normalisation statistics of this training set (FP64 sums)
+    dbuf<double> part;
+    part.alloc((size_t)kStatBlocks * 2 * kNF);
+    for (int k = 0; k < 2; ++k) {
+        const int d = k ? 2 : kNF;
+        GQ_LAUNCH(ctx, k_col_sums, kStatBlocks, 256, 0, n, d, k ? Yd : Xd, part.p);
+        GQ_LAUNCH(ctx, k_col_stats, 1, 32, 0, n, d, (const double *)part, k ? M->ymu.p : M->xmu.p, k ? M->ysd.p : M->xsd.p);
     }
-    GQ_CUDA(cudaMemcpyAsync(M->xmu.p, xmu.data(), sizeof(float) * kNF, cudaMemcpyHostToDevice, st));
-    GQ_CUDA(cudaMemcpyAsync(M->xsd.p, xsd.data(), sizeof(float) * kNF, cudaMemcpyHostToDevice, st));
-    GQ_CUDA(cudaMemcpyAsync(M->ymu.p, ymu.data(), sizeof(float) * 2, cudaMemcpyHostToDevice, st));
-    GQ_CUDA(cudaMemcpyAsync(M->ysd.p, ysd.data(), sizeof(float) * 2, cudaMemcpyHostToDevice, st));
     dbuf<int> permall;
     permall.alloc(n);
     std::vector<int> perm(n);
     for (int i = 0; i < n; ++i) perm[i] = i;
     std::mt19937_64 rng(seed);
-    double last = 0;
     const float b1 = 0.9f, b2 = 0.999f;
+    const int per = gq_blocks(B, kSB);
+    dbuf<double> sse;   // squared errors of the last epoch's batches
+    sse.alloc((size_t)(n / B) * per);
+    GQ_CUDA(cudaMemsetAsync(sse.p, 0, sizeof(double) * (n / B) * per, st));
     for (int ep = 0; ep < epochs; ++ep) {
         std::shuffle(perm.begin(), perm.end(), rng);
         GQ_CUDA(cudaMemcpyAsync(permall.p, perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
-        double sse = 0;
-        for (int s0 = 0; s0 + B <= n; s0 += B) {
-            GQ_LAUNCH(ctx, k_gather_rows, gq_blocks((long long)B * kNF, kT), kT, 0, B, kNF, (const int *)permall.p + s0,
-                      Xd, (const float *)M->xmu.p, (const float *)M->xsd.p, M->Xb.p);
-            GQ_LAUNCH(ctx, k_gather_rows, gq_blocks((long long)B * 2, kT), kT, 0, B, 2, (const int *)permall.p + s0, Yd,
-                      (const float *)M->ymu.p, (const float *)M->ysd.p, M->Yb.p);
-            bool last_batch = ep == epochs - 1;
-            double e = 0;
-            fwd_bwd(M, B, last_batch, &e);
-            sse += e;
+        const bool last_epoch = ep == epochs - 1;
+        for (int s0 = 0, k = 0; s0 + B <= n; s0 += B, ++k) {
             ++M->adam_t;
-            float c1 = 1.f - powf(b1, (float)M->adam_t), c2 = 1.f - powf(b2, (float)M->adam_t);
-            GQ_LAUNCH(ctx, k_adam, gq_blocks(kNParams, kT), kT, 0, kNParams, M->w.p, (const float *)M->g.p, M->m.p,
-                      M->v.p, lr, b1, b2, c1, c2);
+            const float c1 = 1.f - powf(b1, (float)M->adam_t), c2 = 1.f - powf(b2, (float)M->adam_t);
+            mlp_batch(M, B, (const int *)permall + s0, Xd, Yd, true, last_epoch ? sse.p + (size_t)k * per : nullptr,
+                      AdamStep{M->w, M->m, M->v, lr, b1, b2, c1, c2});
         }
-        last = sse / (2.0 * (n / B) * B);
     }
+    const double last = sum_on_host(ctx, sse.p, (size_t)(n / B) * per) / (2.0 * (n / B) * B);
     GQ_CUDA(cudaStreamSynchronize(st));
     return last;   // mean squared error of the last epoch, in normalised units
 }
