@@ -333,7 +333,7 @@ gq_status gq_apply(gq_geom *g, int kernel, double identity, const double *mu, do
             stage.alloc(g->nbase);
             o = stage.p;
         }
-        gq_eval_all(g, kernel, dens, o, nullptr, nullptr, &identity);
+        gq_eval_all(g, kernel, dens, o, nullptr, &identity);
         if (!out_dev) {
             GQ_CUDA(cudaMemcpyAsync(out, o, sizeof(double) * g->nbase, cudaMemcpyDefault, st));
             GQ_CUDA(cudaStreamSynchronize(st));

@@ -123,8 +123,27 @@ __device__ __forceinline__ void warp_reduce_scatter(V (&v)[NV], V zero, int lane
     if (cnt < 0) cnt = 0;
 }
 
+// ------------------------------------------------------------------ multipoles in fixed point
+// exponent of a box whose multipoles are not all finite
+constexpr int kFxNaNExp = 1 << 20;
+static __device__ __forceinline__ double fx_scale_of(int E) {   // 2^(E - 1022)
+    if (E == kFxNaNExp) return __longlong_as_double(0x7ff8000000000000ll);
+    return E + 1 >= 1 ? (E + 1 <= 2046 ? __longlong_as_double((long long)(E + 1) << 52) : 2.0 * __longlong_as_double(2046ll << 52))
+                      : ldexp(1.0, max(E - 1022, -1100));
+}
+
 // direct sums to the QBX centres in 64-bit fixed point (gq_near_fx.cu): Qout [nc][E.Q+1]
 void gq_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double2 *Qout);
+// direct potential at the point targets for S, likewise (gq_near_fx.cu)
+void gq_near_points_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double *pot);
 // List 2 translations (M2L) of orders 16 .. 30 in fixed point (gq_m2l_fx.cu), added to L
 void gq_m2l_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *L);
 void gq_m2l_fx_prepare(int dev);   // its tables on device dev
+// the multipoles of the boxes in fixed point, into g->Mfx and g->Efx (gq_w_fx.cu)
+void gq_mfix(gq_geom *g, int P1, const double2 *M);
+// List 3 far (gq_w_fx.cu), from g->Mfx and g->Efx: multipoles at the point targets, and to
+// the QBX centres for p_qbx <= kWFxMaxQ, added to pot and Q
+constexpr int kWFxMaxQ = 10;
+void gq_w_points_fx(gq_geom *g, const EvalView &E, const double2 *M, double *pot);
+void gq_w_centres_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *Q);
+void gq_w_fx_prepare(int dev);     // its tables on device dev

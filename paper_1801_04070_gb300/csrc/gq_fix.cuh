@@ -139,6 +139,24 @@ GQ_HD long long fx_rcp(uint64_t m) {
     return fx_shl((long long)Y, 40) + (t >> 2);
 }
 
+// u = (re / w) 2^62 from w, |w|^2 = n2 and the radius' significand (R, 2^61) and
+// biased exponent: re / M2 by fx_rcp, each component's significand shifted into
+// the common format (a right shift for |u| < 2), complemented for a negative w (a
+// unit of 2^-62 off) and multiplied.  The lowest bit of u is set so that no low
+// word is -2^31, which has no negative.
+GQ_HD void fx_ratio(double wx, double wy, uint64_t nb, gfx R, int er, gfx &ux, gfx &uy, gfx &nuy) {
+    const gfx G = fx_bal(fx_shl(fx_mul(R, fx_bal(fx_rcp(fx_mant(nb)))), 2));   // 2^61 r / M
+    const int k = er - fx_expo(nb) - 1023 - 1;
+    auto comp = [&](uint64_t b) {
+        const gfx x = fx_bal((long long)fx_shr(fx_mant(b) << 10, -(k + fx_expo(b))) ^ ((long long)b >> 63));
+        return fx_bal(fx_shl(fx_mul(x, G), 4) | 1);
+    };
+    ux = comp(fx_bits(wx));
+    nuy = comp(fx_bits(wy));
+    uy.h = -nuy.h;
+    uy.l = -nuy.l;
+}
+
 // (1/2) log x 2^57 relative to 2^(e_ref - 1023), for the bits of a normal x:
 // Tang's table method (see gq_math.cuh) with t_j a 16-bit integer T_j / 2^16, so
 // that r = m t_j - 1 comes exactly out of the low 64 bits of m T_j; then

@@ -1639,38 +1639,6 @@ __device__ void near_centres_multi_box(const EvalView &E, int b, const double2 *
 }
 
 
-template <int QQ, int KERNEL, int ND>
-__global__ void __launch_bounds__(kNearThreads) k_near_centres_multi(EvalView E, int nwork, const int *__restrict__ work,
-                                                                      const double2 *__restrict__ strm, long long sstride,
-                                                                      double2 *__restrict__ Qm, long long qstride) {
-    __shared__ NearRanges R;
-    __shared__ int wsum[kNearThreads / 32];
-    __shared__ double lt[KERNEL == GQ_D ? 1 : kGqLogN];
-    if (KERNEL != GQ_D)
-        for (int i = threadIdx.x; i < kGqLogN; i += kNearThreads) lt[i] = E.logt[i];
-    near_centres_multi_box<QQ, KERNEL, ND>(E, work[blockIdx.x], strm, sstride, Qm, qstride, R, wsum, lt);
-}
-
-template <int QQ, int ND>
-void launch_near_centres_multi(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, const double2 *strm,
-                               long long sstride, double2 *Qm, long long qstride) {
-    auto kd = k_near_centres_multi<QQ, GQ_D, ND>;
-    auto ks = k_near_centres_multi<QQ, GQ_S, ND>;
-    GQ_LAUNCH(ctx, (E.kernel == GQ_D ? kd : ks), nwork, kNearThreads, 0, E, nwork, work, strm, sstride, Qm, qstride);
-}
-
-template <int ND>
-void dispatch_near_centres_multi(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, const double2 *strm,
-                                 long long sstride, double2 *Qm, long long qstride) {
-    switch (E.Q) {
-#define GQ_CASE(v) case v: launch_near_centres_multi<v, ND>(ctx, E, nwork, work, strm, sstride, Qm, qstride); break;
-        GQ_CASE(1) GQ_CASE(2) GQ_CASE(3) GQ_CASE(4) GQ_CASE(5) GQ_CASE(6) GQ_CASE(7) GQ_CASE(8)
-        GQ_CASE(9) GQ_CASE(10) GQ_CASE(11) GQ_CASE(12) GQ_CASE(13) GQ_CASE(14) GQ_CASE(15) GQ_CASE(16)
-#undef GQ_CASE
-        default: throw gq_error{GQ_ERR_INVALID, "p_qbx out of range"};
-    }
-}
-
 __global__ void k_tgt_ptpos(int npt, const int *__restrict__ pt_perm, int *__restrict__ out) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < npt) out[pt_perm[j]] = j;
@@ -1897,6 +1865,7 @@ static const ConstTables &const_tables(int dev) {
     GqDflLogTable DT;
     gq_dfl_log_table_host(&DT);
     gq_m2l_fx_prepare(dev);
+    gq_w_fx_prepare(dev);
     ConstTables C;
     C.logt = upload_const((const double *)&LT, kGqLogN);
     FxLogTable FT;
@@ -1968,7 +1937,7 @@ static EvalTables &get_tables(gq_geom *g) {
 }
 
 void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev, gq_stats *stt,
-                 const double2 *qn_pre, const double *apply_identity, const EvalFar *far) {
+                 const double *apply_identity, const EvalFar *far) {
     // apply_identity != null: the operator at the base nodes (gq_apply); the
     // point-target stages are skipped and out_dev has one value per base node.
     // far != null: strengths and the FMM passes only, their parts of the QBX
@@ -2117,7 +2086,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         if (f32) dispatch_near_centres_f32(&ctx2, E, X, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
         // the FP32-pair tier too: fixed point is faster than pairs (1.05 M nodes, q = 4: 3.18 ms in pairs) and
         // closer to 64 bits
-        else if (!qn_pre || split) gq_near_centres_fx(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
+        else gq_near_centres_fx(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
     }
     mark(N_CTR, s2);
     if (g->n_pt_boxes && !at_base && !fmm_only) {
@@ -2126,16 +2095,16 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             auto ks = k_near_points_f32<GQ_S>;
             GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, X, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
-        } else if (split) {
+        } else if (split) {   // pairs: 0.72 ms where fixed point takes 1.11 (0.86 M targets)
             auto kd = k_near_points_split<GQ_D>;
             auto ks = k_near_points_split<GQ_S>;
             GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, SX, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
-        } else {
-            auto kd = k_near_points<GQ_D>;
-            auto ks = k_near_points<GQ_S>;
-            GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, g->n_pt_boxes,
+        } else if (kin == GQ_D) {
+            GQ_LAUNCH((&ctx2), k_near_points<GQ_D>, g->n_pt_boxes, kNearThreads, 0, E, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
+        } else {
+            gq_near_points_fx(&ctx2, E, g->n_pt_boxes, g->pt_boxes, g->potn.p);
         }
     }
     mark(N_PT, s2);
@@ -2184,6 +2153,11 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     else if (split_w)   // multipoles as FP32 pairs for the pair List 3 far kernels
         GQ_LAUNCH(ctx, k_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->M, g->M2.p);
+    // the multipoles in fixed point for the kernels that work there
+    const bool m2l_fx = !m2l_split && P1 > 16;
+    const bool wc_fx = !split_w && g->nc > 0 && !gq_w_tc_supported(g) && Qn <= kWFxMaxQ;
+    const bool wp_fx = !f32 && !split_w && g->npt > 0 && !at_base;
+    if (m2l_fx || wc_fx || wp_fx) gq_mfix(g, P1, (const double2 *)g->M);
     // Stage 4
     if (g->n_far_boxes) {
         if (m2l_split) {
@@ -2195,7 +2169,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                       g->n_far_boxes, (const int *)g->far_boxes, T.dtab2, T.logtab2, T.binom2, g->L2.p);
         } else if (gq_m2l_tc_supported(g)) {
             gq_m2l_tc(g, (const double2 *)g->M, g->L.p);   // FP64-accurate, on the tensor cores
-        } else if (P1 > 16) {
+        } else if (m2l_fx) {
             gq_m2l_fx(g, E, (const double2 *)g->M, g->L.p);   // in fixed point
         } else {
             auto k16 = k_m2l<16>;
@@ -2236,6 +2210,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         dispatch_w_centres_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
     } else if (g->nc) {
         if (gq_w_tc_supported(g)) gq_w_centres_tc(g, E.R, (const double2 *)g->M, T.logt, Qb);
+        else if (wc_fx) gq_w_centres_fx(g, E, (const double2 *)g->M, Qb);
         else dispatch_w_centres_q(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
     }
     mark(S_WC, st);
@@ -2247,8 +2222,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             GQ_LAUNCH(ctx, k_w_points_split, gq_blocks(g->npt, 128), 128, 0, E, SX, g->npt, (const int *)g->pt_owner,
                       potb);
         else
-            GQ_LAUNCH(ctx, k_w_points, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner,
-                      (const double2 *)g->M, potb);
+            gq_w_points_fx(g, E, (const double2 *)g->M, potb);
     }
     mark(S_WP, st);
     // Stage 8
@@ -2263,24 +2237,19 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     mark(S_L2Q, st);
     // join the direct part, then evaluate at the targets
     GQ_CUDA(cudaStreamWaitEvent(st, g->ev_near, 0));
-    // the direct part of the QBX coefficients: this call's, or formed beforehand
-    // for several densities at once (gq_eval_multi)
-    const bool use_pre = qn_pre && !f32 && !split;
-    const double2 *qn_use = use_pre ? qn_pre : (const double2 *)g->Qn;
-    g->qn_last = qn_use;
     if (fmm_only) {
         // the direct parts and the final sums are the caller's
     } else if (at_base) {
         if (g->nbase)
             GQ_LAUNCH(ctx, k_final_base, gq_blocks(g->nbase, 256), 256, 0, g->nbase, kernel, Qn, E.qc,
                       (const int *)g->ctr_pos, (const double *)g->base_xy, (const double *)g->base_n,
-                      (const double2 *)g->sc_xy, (const double *)g->sc_r, (const double2 *)g->Q, qn_use,
+                      (const double2 *)g->sc_xy, (const double *)g->sc_r, (const double2 *)g->Q, (const double2 *)g->Qn,
                       *apply_identity, dens_dev, out_dev);
     } else if (g->nt)
         GQ_LAUNCH(ctx, k_final, gq_blocks(g->nt, 256), 256, 0, g->nt, kernel, Qn, E.qc, (const int *)g->t_kind,
                   (const int *)g->t_ctr, (const int *)g->ctr_pos, (const int *)T.tgt_ptpos, (const double *)g->tgt_xy,
                   (const int *)g->tgt_on, (const double *)g->base_n, (const double2 *)g->sc_xy,
-                  (const double *)g->sc_r, (const double2 *)g->Q, qn_use, (const double *)g->pot,
+                  (const double *)g->sc_r, (const double2 *)g->Q, (const double2 *)g->Qn, (const double *)g->pot,
                   (const double *)g->potn, out_dev);
     mark(S_END, st);
     ctx->launches += ctx2.launches;
@@ -2489,7 +2458,7 @@ void gq_bplan_fmm(gq_bplan *P, int i) {
     cudaStream_t st = g->ctx->stream;
     for (int d = 0; d < P->ndens; ++d) {
         EvalFar far{P->Qf[i]->p + (size_t)d * g->nc * Q1, P->potf[i]->p + (size_t)d * (g->npt > 0 ? g->npt : 1)};
-        gq_eval_all(g, P->kernel, P->dens[i] + (size_t)d * g->nbase, nullptr, nullptr, nullptr, nullptr, &far);
+        gq_eval_all(g, P->kernel, P->dens[i] + (size_t)d * g->nbase, nullptr, nullptr, nullptr, &far);
         if (g->nsrc)
             GQ_CUDA(cudaMemcpyAsync(P->strm[i]->p + (size_t)d * g->nsrc, g->strength.p, sizeof(double2) * g->nsrc,
                                     cudaMemcpyDeviceToDevice, st));
@@ -2528,56 +2497,11 @@ int gq_bplan_error(gq_bplan *P) {
     return h;
 }
 
-// Several densities on one geometry: the direct part of the QBX coefficients
-// for all of them by the multi-density kernel (FP64 mode), then the rest of
-// the evaluation per density.  The mixed-precision tiers evaluate one density
-// after another.
+// Several densities on one geometry, one after another: the fixed-point direct
+// sums of four densities cost less than forming the FP64 pair geometry once for
+// all four did.
 void gq_eval_multi(gq_geom *g, int kernel, int nd, const double *const *dens, double *const *out) {
-    const bool mixed = g->prm.precision == GQ_PREC_MIXED || g->prm.precision == GQ_PREC_MIXED_FMM;
-    const bool f32 = mixed && g->prm.eps >= kF32TierEps;
-    const bool split = mixed && g->prm.eps >= 1e-12 && g->prm.eps < kF32TierEps;
-    if (nd <= 1 || f32 || split || g->n_ctr_boxes == 0) {
-        for (int d = 0; d < nd; ++d) gq_eval_all(g, kernel, dens[d], out[d], nullptr);
-        return;
-    }
-    gq_ctx *ctx = g->ctx;
-    EvalTables &T = get_tables(g);
-    int kin = kernel == GQ_SP ? GQ_S : kernel;
-    const int Q1 = g->prm.p_qbx + 1;
-    const long long sstride = g->nsrc, qstride = (long long)g->nc * Q1;
-    g->strm.alloc((size_t)nd * g->nsrc);
-    g->Qm.alloc((size_t)nd * qstride);
-    for (int d = 0; d < nd; ++d)
-        if (g->nsrc)
-            GQ_LAUNCH(ctx, k_strengths, gq_blocks(g->nsrc, 256), 256, 0, g->nsrc, g->nu, g->nb, (const int *)g->src_perm,
-                      (const double *)g->interp, dens[d], (const double *)g->s_w, (const double2 *)g->s_n, kin,
-                      g->strm.p + d * sstride, (unsigned int *)nullptr);
-    EvalView E{};
-    E.R = g->root;
-    E.P = g->prm.p_fmm;
-    E.Q = g->prm.p_qbx;
-    E.kernel = kin;
-    E.blev = g->blev; E.bix = g->bix; E.biy = g->biy; E.bparent = g->bparent; E.bchild = g->bchild;
-    E.src_beg = g->src_beg; E.src_end = g->src_end;
-    E.ctr_beg = g->ctr_beg; E.ctr_end = g->ctr_end; E.pt_beg = g->pt_beg; E.pt_end = g->pt_end;
-    E.sub_src = g->sub_src; E.sub_tgt = g->sub_tgt;
-    E.s_xy = g->s_xy; E.sc_xy = g->sc_xy; E.sc_r = g->sc_r; E.sp_xy = g->sp_xy;
-    for (int i = 0; i < 6; ++i) { E.loff[i] = g->list_off[i]; E.lidx[i] = g->list_idx[i]; }
-    E.binom = T.binom;
-    E.qc = g->has_qc ? (const int *)g->q_ctr.p : nullptr;
-    E.logt = T.logt;
-    E.fxlog = T.fxlog;
-    int d0 = 0;
-    for (; d0 + 4 <= nd; d0 += 4)
-        dispatch_near_centres_multi<4>(ctx, E, g->n_ctr_boxes, g->ctr_boxes, g->strm.p + d0 * sstride, sstride,
-                                       g->Qm.p + d0 * qstride, qstride);
-    for (; d0 + 2 <= nd; d0 += 2)
-        dispatch_near_centres_multi<2>(ctx, E, g->n_ctr_boxes, g->ctr_boxes, g->strm.p + d0 * sstride, sstride,
-                                       g->Qm.p + d0 * qstride, qstride);
-    for (; d0 < nd; ++d0)
-        dispatch_near_centres_multi<1>(ctx, E, g->n_ctr_boxes, g->ctr_boxes, g->strm.p + d0 * sstride, sstride,
-                                       g->Qm.p + d0 * qstride, qstride);
-    for (int d = 0; d < nd; ++d) gq_eval_all(g, kernel, dens[d], out[d], nullptr, g->Qm.p + d * qstride);
+    for (int d = 0; d < nd; ++d) gq_eval_all(g, kernel, dens[d], out[d], nullptr);
 }
 
 void gq_export_qbx_impl(gq_geom *g, double *host) {
@@ -2586,7 +2510,7 @@ void gq_export_qbx_impl(gq_geom *g, double *host) {
     tmp.alloc((size_t)g->nc * Q1);
     GQ_LAUNCH(g->ctx, k_export_qbx, gq_blocks((long long)g->nc * Q1, 256), 256, 0, g->nc, g->prm.p_qbx,
               (const int *)g->ctr_perm, (const double *)g->sc_r, (const double2 *)g->Q,
-              g->qn_last ? g->qn_last : (const double2 *)g->Qn, tmp.p);
+              (const double2 *)g->Qn, tmp.p);
     GQ_CUDA(cudaMemcpyAsync(host, tmp.p, sizeof(double2) * g->nc * Q1, cudaMemcpyDeviceToHost, g->ctx->stream));
     GQ_CUDA(cudaStreamSynchronize(g->ctx->stream));
 }

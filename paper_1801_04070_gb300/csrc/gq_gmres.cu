@@ -71,7 +71,7 @@ struct Solver {
     dbuf<double> hdev;
     void apply(const double *v, double *out) {   // out = -v/2 + S' v at the base nodes (gq_apply)
         const double minus_half = -0.5;
-        gq_eval_all(g, GQ_SP, v, out, nullptr, nullptr, &minus_half);
+        gq_eval_all(g, GQ_SP, v, out, nullptr, &minus_half);
     }
     std::vector<double> dots(const double *V, int k, const double *w) {
         GQ_LAUNCH(g->ctx, k_multidot, k, 1024, 0, n, k, V, w, hdev.p);

@@ -151,7 +151,7 @@ struct gq_geom {
     dbuf<double2> strength;          // sorted sources: S -> (q, 0), D -> d
     dbuf<unsigned int> qexp;         // largest biased exponent of the strengths (one value)
     dbuf<double2> M, L;              // [nbox][p_fmm+1] box-scaled expansions
-    dbuf<int4> Mfx;                  // [nbox][p_fmm+1] multipoles in fixed point (gq_m2l_fx.cu)
+    dbuf<longlong2> Mfx;             // [nbox][p_fmm+1] multipoles in fixed point (gq_w_fx.cu)
     dbuf<int> Efx;                   // [nbox] their exponents
     dbuf<double2> Q;                 // [nc][p_qbx+1] r-scaled QBX coefficients (sorted centres): far part
     dbuf<double2> Qn;                // the same, direct part
@@ -180,9 +180,6 @@ struct gq_geom {
     dbuf<float4> c_rel2;
     dbuf<float4> c_r2;    // (r.hi, r.lo, (1/r^2).hi, (1/r^2).lo)
     dbuf<float4> str2;    // (re.hi, re.lo, im.hi, im.lo)
-    // several densities at once (gq_eval_multi): strengths and direct coefficients per density
-    dbuf<double2> strm, Qm;
-    const double2 *qn_last = nullptr;   // direct coefficients of the last evaluation
     dbuf<float4> p_rel2;  // sorted point targets minus their leaf centre
     dbuf<float4> M2;      // multipoles
     dbuf<float4> L2;      // local expansions
@@ -233,7 +230,7 @@ struct EvalFar {
     double *pot;    // [npt] point potentials from List 3 far and the box locals
 };
 void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev, gq_stats *st,
-                 const double2 *qn_pre = nullptr, const double *apply_identity = nullptr,
+                 const double *apply_identity = nullptr,
                  const EvalFar *far = nullptr);                                            // gq_fmm.cu
 void gq_eval_multi(gq_geom *g, int kernel, int nd, const double *const *dens, double *const *out);
 void gq_export_qbx_impl(gq_geom *g, double *host);  // gq_fmm.cu

@@ -28,36 +28,11 @@
 namespace {
 
 constexpr int kP1 = GQ_MAX_PFMM + 1;
-constexpr int kNaNExp = 1 << 20;   // exponent of a box whose multipoles are not all finite
-
-// Multipoles as fixed point (split at bit 30, [58]) at the box's exponent; a warp
-// per box, lane k an order.
-__global__ void k_mfix(int nbox, int P1, const double2 *__restrict__ M, int4 *__restrict__ Mf, int *__restrict__ Ef) {
-    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, k = threadIdx.x & 31;
-    if (b >= nbox) return;
-    const bool act = k < P1;
-    const double2 A = act ? M[(size_t)b * P1 + k] : make_double2(0.0, 0.0);
-    const int e = max(fx_expo(fx_bits(A.x)), fx_expo(fx_bits(A.y)));
-    const int kc = (k + 1) / 2;
-    const int E = __reduce_max_sync(0xffffffffu, e ? e - kc : -1000);
-    const bool bad = __any_sync(0xffffffffu, e == 0x7ff);
-    if (act) {
-        const gfx30 x = fx_split30(fx_from_double(A.x, E + kc) >> 4), y = fx_split30(fx_from_double(A.y, E + kc) >> 4);
-        Mf[(size_t)b * P1 + k] = make_int4(x.h, x.l, y.h, y.l);
-    }
-    if (k == 0) Ef[b] = bad ? kNaNExp : E;
-}
-
-__device__ __forceinline__ double scale_of(int E) {   // 2^(E - 1022)
-    if (E == kNaNExp) return __longlong_as_double(0x7ff8000000000000ll);
-    return E + 1 >= 1 ? (E + 1 <= 2046 ? __longlong_as_double((long long)(E + 1) << 52) : 2.0 * __longlong_as_double(2046ll << 52))
-                      : ldexp(1.0, max(E - 1022, -1100));
-}
 
 constexpr int kM2LWarps = 4;
 
 __global__ void __launch_bounds__(kM2LWarps * 32) k_m2l_fx(EvalView E, int nwork, const int *__restrict__ work,
-                                                           const double2 *__restrict__ M, const int4 *__restrict__ Mf,
+                                                           const double2 *__restrict__ M, const longlong2 *__restrict__ Mf,
                                                            const int *__restrict__ Ef, const int2 *__restrict__ ctab,
                                                            const int4 *__restrict__ dfix, const double2 *__restrict__ stab,
                                                            const double *__restrict__ logtab, double2 *__restrict__ L) {
@@ -83,9 +58,10 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_m2l_fx(EvalView E, int nwork
                 off[p] = (by - E.biy[d] + 5) * 11 + (bx - E.bix[d] + 5);
                 int4 a4 = make_int4(0, 0, 0, 0);
                 if (act && j + p < end) {
-                    const int4 A = Mf[(size_t)d * P1 + m], D = dfix[off[p] * 32 + m];
+                    const longlong2 A = Mf[(size_t)d * P1 + m];
+                    const int4 D = dfix[off[p] * 32 + m];
                     long long re, im;
-                    fx_cmul30(gfx30{A.x, A.y}, gfx30{A.z, A.w}, gfx{D.x, D.y}, gfx{D.z, D.w}, gfx{-D.z, -D.w}, re, im);
+                    fx_cmul30(fx_split30(A.x), fx_split30(A.y), gfx{D.x, D.y}, gfx{D.z, D.w}, gfx{-D.z, -D.w}, re, im);
                     const gfx x = fx_bal(re), y = fx_bal(im);
                     a4 = make_int4(x.h, x.l, y.h, y.l);
                 }
@@ -109,7 +85,7 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_m2l_fx(EvalView E, int nwork
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 if (j + p >= end) break;
-                const double s = scale_of(Ef[dd[p]]);
+                const double s = fx_scale_of(Ef[dd[p]]);
                 const double2 t = make_double2((double)(hr[p] + (int)(mr[p] >> 32)) * s, (double)(hi[p] + (int)(mi[p] >> 32)) * s);
                 const double2 f = stab[off[p] * 32 + m];
                 // the entry's own terms first: one rounding of the running sum an entry
@@ -205,13 +181,9 @@ const M2LFxTables &tables(int dev) {
 
 void gq_m2l_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *L) {
     const M2LFxTables &T = tables(g->ctx->device);
-    const int P1 = E.P + 1;
-    g->Mfx.alloc((size_t)g->nbox * P1);
-    g->Efx.alloc(g->nbox);
-    GQ_LAUNCH(g->ctx, k_mfix, gq_blocks((long long)g->nbox * 32, 256), 256, 0, g->nbox, P1, M, g->Mfx.p, g->Efx.p);
     const int blocks = gq_blocks(g->n_far_boxes, kM2LWarps);
     GQ_LAUNCH(g->ctx, k_m2l_fx, blocks < 152 * 32 ? blocks : 152 * 32, kM2LWarps * 32, 0, E, g->n_far_boxes,
-              (const int *)g->far_boxes, M, (const int4 *)g->Mfx, (const int *)g->Efx, T.c, T.d, T.s, T.logd, L);
+              (const int *)g->far_boxes, M, (const longlong2 *)g->Mfx, (const int *)g->Efx, T.c, T.d, T.s, T.logd, L);
 }
 
 void gq_m2l_fx_prepare(int dev) { tables(dev); }

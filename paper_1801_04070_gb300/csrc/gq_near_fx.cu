@@ -110,22 +110,72 @@ __device__ __noinline__ void near_centre_slow(const EvalView &E, const NearRange
     }
 }
 
-// u = (re / w) 2^62 from w, |w|^2 = n2 and the radius' significand (R, 2^61) and
-// biased exponent: re / M2 by fx_rcp, each component's significand shifted into
-// the common format (a right shift for |u| < 2), complemented for a negative w (a
-// unit of 2^-62 off) and multiplied.  The lowest bit of u is set so that no low
-// word is -2^31, which has no negative.
-__device__ __forceinline__ void fx_ratio(double wx, double wy, uint64_t nb, gfx R, int er, gfx &ux, gfx &uy, gfx &nuy) {
-    const gfx G = fx_bal(fx_shl(fx_mul(R, fx_bal(fx_rcp(fx_mant(nb)))), 2));   // 2^61 r / M
-    const int k = er - fx_expo(nb) - 1023 - 1;
-    auto comp = [&](uint64_t b) {
-        const gfx x = fx_bal((long long)fx_shr(fx_mant(b) << 10, -(k + fx_expo(b))) ^ ((long long)b >> 63));
-        return fx_bal(fx_shl(fx_mul(x, G), 4) | 1);
-    };
-    ux = comp(fx_bits(wx));
-    nuy = comp(fx_bits(wy));
-    uy.h = -nuy.h;
-    uy.l = -nuy.l;
+// Stage the sources [v0, v1) of the loaded ranges: positions, and strengths as
+// q 2^(1022 - qe) <= 1/2 (D: each component, so that |d| <= 0.36) with qe from the
+// tile's largest exponent; for S the sums of the strengths' words per warp.
+// Returns qe, 0 where the strengths have no scale; ends with a barrier.
+template <int KERNEL>
+__device__ __forceinline__ int fx_stage(const EvalView &E, const NearRanges &R, int v0, int v1, double2 *sy,
+                                        typename FxStr<KERNEL>::T *sq, long long *ssum, int *smax) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int mx = 0;
+    for (int r = w; r < R.n; r += kFxWarps) {   // a warp takes one range at a time
+        const int p0 = R.pre[r], p1 = R.pre[r + 1];
+        for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
+            const double2 st = E.str[R.beg[r] + (v - p0)];
+            mx = max(mx, str_expo(st.x));
+            if (KERNEL == GQ_D) mx = max(mx, str_expo(st.y));
+        }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) smax[w] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kFxWarps; ++k) mx = max(mx, smax[k]);
+    if (mx == 0) mx = 1023;   // all zero
+    const int qe = mx + (KERNEL == GQ_D ? 2 : 1);
+    long long sh = 0, sl = 0;
+    for (int r = w; r < R.n; r += kFxWarps) {
+        const int p0 = R.pre[r], p1 = R.pre[r + 1];
+        for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
+            const int s = R.beg[r] + (v - p0);
+            sy[v - v0] = E.s_xy[s];
+            const double2 st = E.str[s];
+            if constexpr (KERNEL == GQ_D) {
+                const gfx30 a = fx_split30(fx_from_double(st.x, qe + 2));
+                const gfx30 c = fx_split30(fx_from_double(st.y, qe + 2));
+                sq[v - v0] = make_int4(a.h, a.l, c.h, c.l);
+            } else {
+                const gfx a = fx_bal(fx_from_double(st.x, qe));
+                sq[v - v0] = make_int2(a.h, a.l);
+                sh += a.h;
+                sl += a.l;
+            }
+        }
+    }
+    if (KERNEL != GQ_D) {
+        for (int o = 16; o > 0; o >>= 1) {
+            sh += __shfl_xor_sync(0xffffffffu, sh, o);
+            sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        }
+        if (lane == 0) {
+            ssum[2 * w] = sh;
+            ssum[2 * w + 1] = sl;
+        }
+    }
+    __syncthreads();
+    return mx >= 128 && mx <= 1984 ? qe : 0;
+}
+
+// sum of the tile's strengths (2^62 of them) from the warps' words
+__device__ __forceinline__ double fx_strength_sum(const long long *ssum) {
+    long long qh = 0, ql = 0;
+#pragma unroll
+    for (int k = 0; k < kFxWarps; ++k) {
+        qh += ssum[2 * k];
+        ql += ssum[2 * k + 1];
+    }
+    return fma((double)qh, 4294967296.0, (double)ql);
 }
 
 // Blocks an SM is compiled for: the sums take 4 (QQ + 1) registers, and the chains
@@ -165,56 +215,8 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
         for (int v0 = 0; v0 < T || first; v0 += kFxTile) {
             const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
             if (v0) __syncthreads();
-            // the tile's largest strength exponent; strengths are then held as
-            // q 2^(1022 - qe) <= 1/2 (D: each component, so that |d| <= 0.36)
-            int mx = 0;
-            for (int r = w; r < R.n; r += kFxWarps) {
-                const int p0 = R.pre[r], p1 = R.pre[r + 1];
-                for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
-                    const double2 st = E.str[R.beg[r] + (v - p0)];
-                    mx = max(mx, str_expo(st.x));
-                    if (KERNEL == GQ_D) mx = max(mx, str_expo(st.y));
-                }
-            }
-            mx = __reduce_max_sync(0xffffffffu, mx);
-            if (lane == 0) smax[w] = mx;
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < kFxWarps; ++k) mx = max(mx, smax[k]);
-            if (mx == 0) mx = 1023;   // all zero
-            const int qe = mx + (KERNEL == GQ_D ? 2 : 1);
-            const bool scaled = mx >= 128 && mx <= 1984;
-            // stage the tile: a warp copies one range at a time
-            long long sh = 0, sl = 0;
-            for (int r = w; r < R.n; r += kFxWarps) {
-                const int p0 = R.pre[r], p1 = R.pre[r + 1];
-                for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
-                    const int s = R.beg[r] + (v - p0);
-                    sy[v - v0] = E.s_xy[s];
-                    const double2 st = E.str[s];
-                    if constexpr (KERNEL == GQ_D) {
-                        const gfx30 a = fx_split30(fx_from_double(st.x, qe + 2));
-                        const gfx30 c = fx_split30(fx_from_double(st.y, qe + 2));
-                        sq[v - v0] = make_int4(a.h, a.l, c.h, c.l);
-                    } else {
-                        const gfx a = fx_bal(fx_from_double(st.x, qe));
-                        sq[v - v0] = make_int2(a.h, a.l);
-                        sh += a.h;
-                        sl += a.l;
-                    }
-                }
-            }
-            if (KERNEL != GQ_D) {
-                for (int o = 16; o > 0; o >>= 1) {
-                    sh += __shfl_xor_sync(0xffffffffu, sh, o);
-                    sl += __shfl_xor_sync(0xffffffffu, sl, o);
-                }
-                if (lane == 0) {
-                    ssum[2 * w] = sh;
-                    ssum[2 * w + 1] = sl;
-                }
-            }
-            __syncthreads();
+            const int qe = fx_stage<KERNEL>(E, R, v0, v1, sy, sq, ssum, smax);
+            const bool scaled = qe > 0;
             for (int c = cb + w; c < ce; c += kFxWarps) {
                 const double2 cz = E.sc_xy[c];
                 const double rc = E.sc_r[c];
@@ -318,14 +320,8 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                         if (KERNEL != GQ_D && m == 0) {
                             x = 0.0;
                             if (i == 0) {
-                                long long qh = 0, ql = 0;
-#pragma unroll
-                                for (int k = 0; k < kFxWarps; ++k) {
-                                    qh += ssum[2 * k];
-                                    ql += ssum[2 * k + 1];
-                                }
-                                // sum q (2^62) = qh 2^32 + ql; the log terms have 2^55
-                                const double sumq = fma((double)qh, 4294967296.0, (double)ql);
+                                // the log terms have 2^55, the strengths 2^62
+                                const double sumq = fx_strength_sum(ssum);
                                 x = fma((double)acc[0], 134217728.0, (double)lo) * sc +
                                     sumq * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264);
                             }
@@ -338,6 +334,88 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                         }
                         d[i] = first ? x : d[i] + x;
                     }
+            }
+            first = false;
+        }
+    }
+}
+
+// Potential at the point targets for S, sum q log|t - y| (coincident sources
+// skipped): a block per target box, a warp per target, lanes stride over the
+// staged sources; |w|^2 in FP64 (four instructions of the 12.7 that the FP64 form
+// took a pair, which bound it), logarithm, products and sums in fixed point.  What
+// bounds it now is the latency of a box's short work (about ten targets and 70
+// sources): resident blocks over several boxes 1.3 ms, without staging 1.5, a warp a
+// box 1.8, a warp per eight targets 1.6.  0.86 M point targets: 1.37 -> 1.11 ms, 0.20 M:
+// 0.53 -> 0.37.
+__global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, const int *__restrict__ work,
+                                                                 double *__restrict__ pot) {
+    __shared__ NearRanges R;
+    __shared__ int wsum[kFxWarps];
+    __shared__ double2 sy[kFxTile];
+    __shared__ int2 sq[kFxTile];
+    __shared__ long long shl_[kFxLogJ];
+    __shared__ int stj[kFxLogJ];
+    __shared__ long long ssum[2 * kFxWarps];
+    __shared__ int smax[kFxWarps];
+    for (int i = threadIdx.x; i < kFxLogJ; i += kNearThreads) {
+        shl_[i] = E.fxlog->hl[i];
+        stj[i] = E.fxlog->t[i];
+    }
+    const int b = work[blockIdx.x];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ne = (E.loff[0][b + 1] - E.loff[0][b]) + (E.loff[2][b + 1] - E.loff[2][b]) + (E.loff[4][b + 1] - E.loff[4][b]);
+    const int tb = E.pt_beg[b], te = E.pt_end[b];
+    const int eref = 2 * fx_expo(fx_bits(box_rho(E.R, E.blev[b]))) - 1023;   // logarithms relative to rho^2
+    bool first = true;
+    for (int e0 = 0; e0 < ne || first; e0 += kNearRanges) {
+        __syncthreads();
+        load_ranges(E, b, e0, ne, R, wsum);
+        const int T = R.pre[R.n];
+        for (int v0 = 0; v0 < T || first; v0 += kFxTile) {
+            const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
+            if (v0) __syncthreads();
+            const int qe = fx_stage<GQ_S>(E, R, v0, v1, sy, sq, ssum, smax);
+            for (int t = tb + w; t < te; t += kFxWarps) {
+                const double2 tz = E.sp_xy[t];
+                long long acc = 0;
+                unsigned nmin = 0xffffffffu, nmax = 0;
+                if (qe > 0)
+                    for (int v = lane; v < n; v += 32) {
+                        const double2 y = sy[v];
+                        const double wx = y.x - tz.x, wy = y.y - tz.y;
+                        const uint64_t nb = fx_bits(fma(wx, wx, wy * wy));
+                        nmin = min(nmin, (unsigned)(nb >> 32));
+                        nmax = max(nmax, (unsigned)(nb >> 32));
+                        const int2 sv = sq[v];
+                        acc += fx_mul(gfx{sv.x, sv.y}, fx_bal(fx_log_half(nb, eref, shl_, stj)));
+                    }
+                nmin = __reduce_min_sync(0xffffffffu, nmin);
+                nmax = __reduce_max_sync(0xffffffffu, nmax);
+                const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20);
+                double x;
+                if (qe > 0 && (n == 0 || (emin >= 128 && emax <= 1920 && emax - eref <= 40 && eref - emin <= 40))) {
+                    // 12 terms below 2^58.8 a lane: the sum over lanes in two words
+                    int lo = (int)(acc & ((1 << 24) - 1));
+                    long long hi = acc >> 24;
+                    for (int o = 16; o > 0; o >>= 1) hi += __shfl_xor_sync(0xffffffffu, hi, o);
+                    lo = __reduce_add_sync(0xffffffffu, lo);
+                    const double sc = pow2_clamped(qe + 1 - 55);
+                    x = fma((double)hi, 16777216.0, (double)lo) * sc +
+                        fx_strength_sum(ssum) * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264);
+                } else {   // in FP64, infinities and coincident sources included
+                    x = 0.0;
+                    int r = 0;
+                    for (int v = v0 + lane; v < v1; v += 32) {
+                        while (R.pre[r + 1] <= v) ++r;
+                        const int s = R.beg[r] + (v - R.pre[r]);
+                        const double2 y = E.s_xy[s];
+                        const double wx = y.x - tz.x, wy = y.y - tz.y, n2 = wx * wx + wy * wy;
+                        x = fma(E.str[s].x, n2 == 0.0 ? 0.0 : gq_log_half(n2, E.logt), x);
+                    }
+                    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                }
+                if (lane == 0) pot[t] = first ? x : pot[t] + x;
             }
             first = false;
         }
@@ -361,4 +439,8 @@ void gq_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *wo
 #undef GQ_CASE
         default: throw gq_error{GQ_ERR_INVALID, "p_qbx out of range"};
     }
+}
+
+void gq_near_points_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double *pot) {
+    GQ_LAUNCH(ctx, k_near_points_fx, nwork, kNearThreads, 0, E, work, pot);
 }

@@ -161,3 +161,34 @@ def test_list2_in_fixed_point(p):
         torch.cuda.synchronize()
         assert (a - b).abs().max().item() <= 1e-13 * b.abs().max().item(), kern
     geo.close()
+
+
+@pytest.mark.parametrize("p,q", [(1, 1), (2, 3), (15, 16), (17, 4), (18, 10), (30, 7)])
+def test_list3_far_in_fixed_point(p, q):
+    """List 3 far at the point targets (k_w_points_fx; odd and even orders) and to
+    the centres where the tensor cores do not take it (k_w_centres_fx, p_fmm > 16),
+    and the direct sums at the point targets (k_near_points_fx), against the FP64
+    kernels of the no-allocation evaluation; the bound as for List 2."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import ctypes as C
+
+    from paper_1801_04070_gb300 import Geometry, params_default
+    from paper_1801_04070_gb300 import _lib
+    g = workloads.small_grid(2, 2, 20, 4000, seed=p + q)
+    geo = Geometry(g, params_default(p_qbx=q, p_fmm=p, n_max=32))
+    geo.build()
+    assert geo.info.list_size[3] > 1000 and geo.npt > 100
+    dens = torch.tensor(g["density"], dtype=torch.float64, device="cuda")
+    for kern in ("S", "D"):
+        a = torch.empty(geo.nt, dtype=torch.float64, device="cuda")
+        b = torch.empty_like(a)
+        geo.eval(kern, dens, a)
+        geo._check(geo.L.gq_eval_noalloc(geo._geom, _lib.KERNELS[kern], C.c_void_p(dens.data_ptr()), C.c_void_p(b.data_ptr())))
+        torch.cuda.synchronize()
+        pts = torch.tensor(geo.association()[0] == 0, device="cuda")
+        assert (a - b)[pts].abs().max().item() <= 1e-13 * b.abs().max().item(), kern
+        # inside-disk sources of these coarse panels amplify the direct sums' rounding by |r/w|^q
+        assert (a - b).abs().max().item() <= 1e-13 * b.abs().max().item() * 4.0 ** max(0, q - 5), kern
+    geo.close()
