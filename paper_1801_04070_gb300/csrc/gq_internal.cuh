@@ -196,6 +196,7 @@ struct gq_geom {
     dbuf<int> tc_tile_box, tc_slot_src, tc_tile_q, tc_err, tc_lexp, tc_counter, tc_ntiles_dev, tc_cnt;
     dbuf<unsigned> tc_tile_mask;
     dbuf<uint16_t> tc_mdig;
+    dbuf<unsigned long long> tc_part;   // sums of the parts of split tiles
 };
 
 // ------------------------------------------------------------------ launch helpers
