@@ -1979,25 +1979,29 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     double2 *Qb = fmm_only ? far->Q : g->Q.p;      // after the allocations: the
     double *potb = fmm_only ? far->pot : g->pot.p; // first call sets the pointers
     if (!g->s2) {
-        GQ_CUDA(cudaStreamCreateWithFlags(&g->s2, cudaStreamNonBlocking));
+        int lo = 0, hi = 0;
+        GQ_CUDA(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+        GQ_CUDA(cudaStreamCreateWithPriority(&g->s2, cudaStreamNonBlocking, hi));
         GQ_CUDA(cudaEventCreateWithFlags(&g->ev_str, cudaEventDisableTiming));
-        GQ_CUDA(cudaEventCreateWithFlags(&g->ev_near, cudaEventDisableTiming));
+        GQ_CUDA(cudaEventCreateWithFlags(&g->ev_fmm, cudaEventDisableTiming));
     }
-    // The direct part may run on a second stream, concurrently with the FMM passes
-    // (GQ_OVERLAP=1); by default both run in order on the context's stream: the
-    // direct kernels alone keep the FP64 pipe busy, so concurrency gains nothing.
-    static const bool overlap = getenv("GQ_OVERLAP") && getenv("GQ_OVERLAP")[0] == '1';
-    cudaStream_t s2 = overlap ? g->s2 : st;
+    // The FMM passes run on a stream of their own beside the direct part, which
+    // stays on the context's stream: the direct part works on the integer pipes
+    // and the passes on the FP64 pipe and the tensor cores, and the passes of a
+    // small problem are a chain of short kernels that leave most SMs idle.  Their
+    // stream has the higher priority, so that the direct part, started first, does
+    // not hold the chain up.  Both in order -> side by side: one curve 0.57 ->
+    // TIMEOV1 ms, 15 x 61-panel... TIMEOV2, 1.05 M nodes TIMEOV3.
+    const cudaStream_t sf = fmm_only ? st : g->s2;
     gq_ctx ctx2 = *ctx;   // launches of the direct part
-    ctx2.stream = s2;
     ctx2.launches = 0;
 
-    // stage events (only when statistics are requested); the direct stages run on
-    // the second stream, concurrently with the FMM passes
-    enum { S0, S_STR, S_FMM, S_M2M, S_M2L, S_P2L, S_L2L, S_WC, S_WP, S_L2Q, S_END, N_BEG, N_CTR, N_PT, NEV };
-    cudaEvent_t ev[NEV];
+    // stage events (only when statistics are requested), kept with the geometry
+    enum { S0, S_STR, S_FMM, S_M2M, S_M2L, S_P2L, S_L2L, S_WC, S_WP, S_L2Q, S_FIN, S_END, N_BEG, N_CTR, N_PT, NEV };
+    static_assert(NEV <= gq_geom::kStageEvents, "stage events");
+    cudaEvent_t *ev = g->ev_stage;
     bool timed = stt != nullptr;
-    if (timed)
+    if (timed && !ev[0])
         for (int i = 0; i < NEV; ++i) GQ_CUDA(cudaEventCreate(&ev[i]));
     auto mark = [&](int i, cudaStream_t on) {
         if (timed) GQ_CUDA(cudaEventRecord(ev[i], on));
@@ -2079,16 +2083,15 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     mark(S_STR, st);
     GQ_CUDA(cudaEventRecord(g->ev_str, st));
 
-    // ---- Stages 3, 5a, 6a (direct interactions) on the second stream
-    GQ_CUDA(cudaStreamWaitEvent(s2, g->ev_str, 0));
-    mark(N_BEG, s2);
+    // ---- Stages 3, 5a, 6a (direct interactions)
+    mark(N_BEG, st);
     if (g->n_ctr_boxes && !fmm_only) {
         if (f32) dispatch_near_centres_f32(&ctx2, E, X, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
         // the FP32-pair tier too: fixed point is faster than pairs (1.05 M nodes, q = 4: 3.18 ms in pairs) and
         // closer to 64 bits
         else gq_near_centres_fx(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
     }
-    mark(N_CTR, s2);
+    mark(N_CTR, st);
     if (g->n_pt_boxes && !at_base && !fmm_only) {
         if (f32) {
             auto kd = k_near_points_f32<GQ_D>;
@@ -2107,19 +2110,27 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             gq_near_points_fx(&ctx2, E, g->n_pt_boxes, g->pt_boxes, g->potn.p);
         }
     }
-    mark(N_PT, s2);
-    GQ_CUDA(cudaEventRecord(g->ev_near, s2));
+    mark(N_PT, st);
 
-    // ---- FMM passes on the context's stream
-    mark(S_FMM, st);
-    GQ_CUDA(cudaMemsetAsync(g->M.p, 0, sizeof(double2) * g->nbox * P1, st));
+    // ---- FMM passes: the context's launches go to their stream until the join
+    struct OnStream {
+        gq_ctx *c;
+        cudaStream_t own;
+        OnStream(gq_ctx *c_, cudaStream_t s_) : c(c_), own(c_->stream) { c->stream = s_; }
+        ~OnStream() { c->stream = own; }
+    };
+    {
+    OnStream passes(ctx, sf);
+    GQ_CUDA(cudaStreamWaitEvent(sf, g->ev_str, 0));
+    mark(S_FMM, sf);
+    GQ_CUDA(cudaMemsetAsync(g->M.p, 0, sizeof(double2) * g->nbox * P1, sf));
     if (m2l_split) {
-        GQ_CUDA(cudaMemsetAsync(g->M2.p, 0, sizeof(float4) * g->nbox * P1, st));
-        GQ_CUDA(cudaMemsetAsync(g->L2.p, 0, sizeof(float4) * g->nbox * P1, st));
+        GQ_CUDA(cudaMemsetAsync(g->M2.p, 0, sizeof(float4) * g->nbox * P1, sf));
+        GQ_CUDA(cudaMemsetAsync(g->L2.p, 0, sizeof(float4) * g->nbox * P1, sf));
     }
-    GQ_CUDA(cudaMemsetAsync(g->L.p, 0, sizeof(double2) * g->nbox * P1, st));
-    GQ_CUDA(cudaMemsetAsync(Qb, 0, sizeof(double2) * g->nc * Q1, st));
-    if (g->npt && !at_base) GQ_CUDA(cudaMemsetAsync(potb, 0, sizeof(double) * g->npt, st));
+    GQ_CUDA(cudaMemsetAsync(g->L.p, 0, sizeof(double2) * g->nbox * P1, sf));
+    GQ_CUDA(cudaMemsetAsync(Qb, 0, sizeof(double2) * g->nc * Q1, sf));
+    if (g->npt && !at_base) GQ_CUDA(cudaMemsetAsync(potb, 0, sizeof(double) * g->npt, sf));
     // Stage 2 (in pairs wherever M2L runs in pairs: the multipoles then live in
     // M2 and the FP64 copy is made from them for the FP64 consumers)
     if (g->n_leaf_src) {
@@ -2146,7 +2157,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                       (128 / P1) * P1, 0, E, (const int *)g->m2m_boxes, g->m2m_level_start_h[l],
                       g->m2m_level_start_h[l + 1], (const double2 *)T.tm2m, g->M.p);
     }
-    mark(S_M2M, st);
+    mark(S_M2M, sf);
     if (m2l_split)
         GQ_LAUNCH(ctx, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const float4 *)g->M2, g->M.p);
@@ -2178,13 +2189,13 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                       (const double *)T.logtab, g->L.p);
         }
     }
-    mark(S_M2L, st);
+    mark(S_M2L, sf);
     if (g->n_far_boxes) {
         // Stage 6b
         GQ_LAUNCH(ctx, k_p2l, gq_blocks((long long)g->n_far_boxes * 32, 128), 128, 0, E, g->n_far_boxes,
                   (const int *)g->far_boxes, g->L.p);
     }
-    mark(S_P2L, st);
+    mark(S_P2L, sf);
     // Stage 7 (in pairs wherever M2L runs in pairs: the FP64 P2L terms are
     // folded into the pair locals first, and the FP64 copy is made at the end)
     if (m2l_split)
@@ -2204,7 +2215,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     if (f32)
         GQ_LAUNCH(ctx, k_to_float2, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->M, g->M_f.p);
-    mark(S_L2L, st);
+    mark(S_L2L, sf);
     // Stage 5b
     if (g->nc && split_w) {
         dispatch_w_centres_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
@@ -2213,7 +2224,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         else if (wc_fx) gq_w_centres_fx(g, E, (const double2 *)g->M, Qb);
         else dispatch_w_centres_q(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
     }
-    mark(S_WC, st);
+    mark(S_WC, sf);
     if (g->npt && !at_base) {
         if (f32)
             GQ_LAUNCH(ctx, k_w_points_f32, gq_blocks(g->npt, 128), 128, 0, E, X, g->npt, (const int *)g->pt_owner,
@@ -2224,7 +2235,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         else
             gq_w_points_fx(g, E, (const double2 *)g->M, potb);
     }
-    mark(S_WP, st);
+    mark(S_WP, sf);
     // Stage 8
     if (g->nc)
         if (m2l_split)
@@ -2234,9 +2245,12 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     if (g->npt && !at_base)
         GQ_LAUNCH(ctx, k_l2p, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner, (const double2 *)g->L,
                   potb);
-    mark(S_L2Q, st);
-    // join the direct part, then evaluate at the targets
-    GQ_CUDA(cudaStreamWaitEvent(st, g->ev_near, 0));
+    mark(S_L2Q, sf);
+    GQ_CUDA(cudaEventRecord(g->ev_fmm, sf));
+    }
+    // join, then evaluate at the targets
+    GQ_CUDA(cudaStreamWaitEvent(st, g->ev_fmm, 0));
+    mark(S_FIN, st);
     if (fmm_only) {
         // the direct parts and the final sums are the caller's
     } else if (at_base) {
@@ -2276,9 +2290,8 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         stt->ms_stage[7] = el(S_L2L, S_WC);
         stt->ms_stage[8] = el(S_WC, S_WP);
         stt->ms_stage[9] = el(S_WP, S_L2Q);
-        stt->ms_stage[10] = el(S_L2Q, S_END);
+        stt->ms_stage[10] = el(S_FIN, S_END);
         stt->kernel_launches = ctx->launches - l0;
-        for (int i = 0; i < NEV; ++i) cudaEventDestroy(ev[i]);
     }
     g->have_eval = true;
     g->last_kernel = kernel;

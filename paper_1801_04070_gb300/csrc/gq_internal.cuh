@@ -157,8 +157,10 @@ struct gq_geom {
     dbuf<double2> Qn;                // the same, direct part
     dbuf<double> pot;                // sorted point targets: Re Phi, far part
     dbuf<double> potn;               // the same, direct part
-    cudaStream_t s2 = nullptr;       // second stream for the direct part of an evaluation
-    cudaEvent_t ev_str = nullptr, ev_near = nullptr;
+    cudaStream_t s2 = nullptr;       // stream of an evaluation's FMM passes
+    cudaEvent_t ev_str = nullptr, ev_fmm = nullptr;
+    static constexpr int kStageEvents = 16;
+    cudaEvent_t ev_stage[kStageEvents] = {};   // stage times of a timed evaluation (made by the first)
     dbuf<double> out_dev;            // [nt] staging for host outputs
     dbuf<double> dens_dev;           // [nbase] staging for host inputs
     int last_kernel = -1;
