@@ -220,6 +220,8 @@ gq_status gq_geometry_destroy(gq_geom *g) {
         cudaStreamSynchronize(g->s2);
         cudaStreamDestroy(g->s2);
         cudaEventDestroy(g->ev_str);
+        cudaEventDestroy(g->ev_m2m);
+        cudaEventDestroy(g->ev_w);
         cudaEventDestroy(g->ev_fmm);
         for (cudaEvent_t e : g->ev_stage)
             if (e) cudaEventDestroy(e);

@@ -1984,6 +1984,8 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         GQ_CUDA(cudaStreamCreateWithPriority(&g->s2, cudaStreamNonBlocking, hi));
         GQ_CUDA(cudaEventCreateWithFlags(&g->ev_str, cudaEventDisableTiming));
         GQ_CUDA(cudaEventCreateWithFlags(&g->ev_fmm, cudaEventDisableTiming));
+        GQ_CUDA(cudaEventCreateWithFlags(&g->ev_m2m, cudaEventDisableTiming));
+        GQ_CUDA(cudaEventCreateWithFlags(&g->ev_w, cudaEventDisableTiming));
     }
     // The FMM passes run on a stream of their own beside the direct part, which
     // stays on the context's stream: the direct part works on the integer pipes
@@ -1992,12 +1994,21 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // stream has the higher priority, so that the direct part, started first, does
     // not hold the chain up.  Both in order -> side by side: one curve 0.57 ->
     // TIMEOV1 ms, 15 x 61-panel... TIMEOV2, 1.05 M nodes TIMEOV3.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GQ_CUDA(cudaStreamIsCapturing(st, &cap));
     const cudaStream_t sf = fmm_only ? st : g->s2;
+    // List 3 far needs only the multipoles: it follows the direct part on the
+    // context's stream, so that a chain of M2L, L2L and Stage 8 is left (35 curves
+    // 1.89 -> 1.73 ms).  Where the direct part is the longer of the two it follows
+    // M2L and L2L instead (1.05 M nodes, mixed tier: 8.86 -> 8.70), and in a captured
+    // graph of many evaluations (12 geometries x 8 densities 35 -> 26 ms).  Either way
+    // Stage 8 adds to its sums.
+    const bool w_beside = !fmm_only && cap == cudaStreamCaptureStatusNone && g->nsrc < 800000;
     gq_ctx ctx2 = *ctx;   // launches of the direct part
     ctx2.launches = 0;
 
     // stage events (only when statistics are requested), kept with the geometry
-    enum { S0, S_STR, S_FMM, S_M2M, S_M2L, S_P2L, S_L2L, S_WC, S_WP, S_L2Q, S_FIN, S_END, N_BEG, N_CTR, N_PT, NEV };
+    enum { S0, S_STR, S_FMM, S_M2M, S_M2L, S_P2L, S_L2L, S_S8, S_L2Q, S_WB, S_WC, S_WP, S_FIN, S_END, N_BEG, N_CTR, N_PT, NEV };
     static_assert(NEV <= gq_geom::kStageEvents, "stage events");
     cudaEvent_t *ev = g->ev_stage;
     bool timed = stt != nullptr;
@@ -2112,6 +2123,34 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     }
     mark(N_PT, st);
 
+    // which stages run in fixed point
+    const bool m2l_fx = !m2l_split && P1 > 16;
+    const bool wc_fx = !split_w && g->nc > 0 && !gq_w_tc_supported(g) && Qn <= kWFxMaxQ;
+    const bool wp_fx = !f32 && !split_w && g->npt > 0 && !at_base;
+    // Stage 5b, on the stream that the context's launches go to
+    auto list3_far = [&]() {
+        mark(S_WB, ctx->stream);
+        if (g->nc && split_w) {
+            dispatch_w_centres_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
+        } else if (g->nc) {
+            if (gq_w_tc_supported(g)) gq_w_centres_tc(g, E.R, (const double2 *)g->M, T.logt, Qb);
+            else if (wc_fx) gq_w_centres_fx(g, E, (const double2 *)g->M, Qb);
+            else dispatch_w_centres_q(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
+        }
+        mark(S_WC, ctx->stream);
+        if (g->npt && !at_base) {
+            if (f32)
+                GQ_LAUNCH(ctx, k_w_points_f32, gq_blocks(g->npt, 128), 128, 0, E, X, g->npt, (const int *)g->pt_owner,
+                          potb);
+            else if (split_w)
+                GQ_LAUNCH(ctx, k_w_points_split, gq_blocks(g->npt, 128), 128, 0, E, SX, g->npt, (const int *)g->pt_owner,
+                          potb);
+            else
+                gq_w_points_fx(g, E, (const double2 *)g->M, potb);
+        }
+        mark(S_WP, ctx->stream);
+    };
+
     // ---- FMM passes: the context's launches go to their stream until the join
     struct OnStream {
         gq_ctx *c;
@@ -2165,10 +2204,11 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         GQ_LAUNCH(ctx, k_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->M, g->M2.p);
     // the multipoles in fixed point for the kernels that work there
-    const bool m2l_fx = !m2l_split && P1 > 16;
-    const bool wc_fx = !split_w && g->nc > 0 && !gq_w_tc_supported(g) && Qn <= kWFxMaxQ;
-    const bool wp_fx = !f32 && !split_w && g->npt > 0 && !at_base;
     if (m2l_fx || wc_fx || wp_fx) gq_mfix(g, P1, (const double2 *)g->M);
+    if (f32)
+        GQ_LAUNCH(ctx, k_to_float2, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+                  (const double2 *)g->M, g->M_f.p);
+    GQ_CUDA(cudaEventRecord(g->ev_m2m, sf));
     // Stage 4
     if (g->n_far_boxes) {
         if (m2l_split) {
@@ -2212,30 +2252,18 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     if (m2l_split)
         GQ_LAUNCH(ctx, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const float4 *)g->L2, g->L.p);
-    if (f32)
-        GQ_LAUNCH(ctx, k_to_float2, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
-                  (const double2 *)g->M, g->M_f.p);
     mark(S_L2L, sf);
-    // Stage 5b
-    if (g->nc && split_w) {
-        dispatch_w_centres_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
-    } else if (g->nc) {
-        if (gq_w_tc_supported(g)) gq_w_centres_tc(g, E.R, (const double2 *)g->M, T.logt, Qb);
-        else if (wc_fx) gq_w_centres_fx(g, E, (const double2 *)g->M, Qb);
-        else dispatch_w_centres_q(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
+    if (w_beside) {
+        ctx->stream = st;
+        GQ_CUDA(cudaStreamWaitEvent(st, g->ev_m2m, 0));
+        list3_far();
+        GQ_CUDA(cudaEventRecord(g->ev_w, st));
+        ctx->stream = sf;
+        GQ_CUDA(cudaStreamWaitEvent(sf, g->ev_w, 0));
+    } else {
+        list3_far();
     }
-    mark(S_WC, sf);
-    if (g->npt && !at_base) {
-        if (f32)
-            GQ_LAUNCH(ctx, k_w_points_f32, gq_blocks(g->npt, 128), 128, 0, E, X, g->npt, (const int *)g->pt_owner,
-                      potb);
-        else if (split_w)
-            GQ_LAUNCH(ctx, k_w_points_split, gq_blocks(g->npt, 128), 128, 0, E, SX, g->npt, (const int *)g->pt_owner,
-                      potb);
-        else
-            gq_w_points_fx(g, E, (const double2 *)g->M, potb);
-    }
-    mark(S_WP, sf);
+    mark(S_S8, sf);
     // Stage 8
     if (g->nc)
         if (m2l_split)
@@ -2287,9 +2315,9 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         stt->ms_stage[4] = el(S_P2L, S_L2L);
         stt->ms_stage[5] = el(N_BEG, N_CTR);
         stt->ms_stage[6] = el(N_CTR, N_PT);
-        stt->ms_stage[7] = el(S_L2L, S_WC);
+        stt->ms_stage[7] = el(S_WB, S_WC);
         stt->ms_stage[8] = el(S_WC, S_WP);
-        stt->ms_stage[9] = el(S_WP, S_L2Q);
+        stt->ms_stage[9] = el(S_S8, S_L2Q);
         stt->ms_stage[10] = el(S_FIN, S_END);
         stt->kernel_launches = ctx->launches - l0;
     }

@@ -158,8 +158,8 @@ struct gq_geom {
     dbuf<double> pot;                // sorted point targets: Re Phi, far part
     dbuf<double> potn;               // the same, direct part
     cudaStream_t s2 = nullptr;       // stream of an evaluation's FMM passes
-    cudaEvent_t ev_str = nullptr, ev_fmm = nullptr;
-    static constexpr int kStageEvents = 16;
+    cudaEvent_t ev_str = nullptr, ev_m2m = nullptr, ev_w = nullptr, ev_fmm = nullptr;
+    static constexpr int kStageEvents = 20;
     cudaEvent_t ev_stage[kStageEvents] = {};   // stage times of a timed evaluation (made by the first)
     dbuf<double> out_dev;            // [nt] staging for host outputs
     dbuf<double> dens_dev;           // [nbase] staging for host inputs
