@@ -49,3 +49,55 @@ def test_standardisation_and_training_reduce_the_error():
     assert np.isfinite(p).all() and ((p - Y) ** 2).mean() < 0.5 * Y.var()
     m.close()
     geo.close()
+
+
+def _features_reference(geo, g):
+    """The features straight from their definition, on the host: every source of
+    the centre's direct lists measured, panels in order of their nearest source
+    (of equal FP32 distances, the one whose source comes first in the lists)."""
+    bx, L = geo.boxes(), geo.lists()
+    so, co, _ = geo.owners()
+    xy, r, _ = geo.centres()
+    srcs = [np.nonzero(so == b)[0] for b in range(geo.nbox)]
+    nu = g["nu"]
+    # sources of a leaf in the library's order: any order gives the same minima
+    out = np.zeros((geo.nc, 16), np.float32)
+    for c in range(geo.nc):
+        b = co[c]
+        near = np.concatenate([srcs[d] for n in ("U", "WC", "XC") for d in L[n][1][L[n][0][b]:L[n][0][b + 1]]] + [np.zeros(0, int)])
+        near = near[near // nu != c // 2 // g["nb"]]
+        dist = (np.hypot(g["up_xy"][near, 0] - xy[c, 0], g["up_xy"][near, 1] - xy[c, 1]) / r[c]).astype(np.float32)
+        best = {}
+        for p, d in zip((near // nu).tolist(), dist.tolist()):
+            best[p] = min(best.get(p, np.inf), d)
+        top = sorted(best.items(), key=lambda t: t[1])[:8]
+        own = g["panel_len"][c // 2 // g["nb"]]
+        out[c, :8] = [min(d, 64.0) for _, d in top] + [64.0] * (8 - len(top))
+        out[c, 8:] = [g["panel_len"][p] / own for p, _ in top] + [0.0] * (8 - len(top))
+    return out
+
+
+@pytest.mark.parametrize("n_max,panels", [(32, 24), (2, 12), (4000, 20), (4000, 140)])
+def test_nearest_panel_features(n_max, panels):
+    """Boxes with few and with many sources (4,000 staged at most; one box holding
+    two curves of 140 panels has 17,920 and takes a thread per centre)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import workloads
+    from paper_1801_04070_gb300 import Geometry, params_default
+    g = workloads.small_grid(2, 1, panels, 50, seed=5)
+    if panels == 140:
+        n_max = 100000
+    geo = Geometry(g, params_default(p_qbx=4, p_fmm=8, n_max=n_max))
+    geo.build()
+    f = geo.features()
+    ref = _features_reference(geo, g) if panels < 100 else None
+    if ref is not None:
+        # distances: one rounding of the hypotenuse and one of the division (2 ulp of FP64) before FP32
+        assert np.abs(f[:, :8] - ref[:, :8]).max() <= 64 * 2.0 ** -23
+        same = np.abs(np.diff(ref[:, :8], axis=1)).min(1) > 1e-5   # no ties: the order is certain
+        assert np.array_equal(f[same, 8:16], ref[same, 8:16]) and same.mean() > 0.5
+    else:
+        assert np.isfinite(f).all() and (np.diff(f[:, :8], axis=1) >= 0).all() and (f[:, 0] > 0).all()
+    geo.close()
