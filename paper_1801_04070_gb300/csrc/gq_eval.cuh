@@ -147,3 +147,6 @@ constexpr int kWFxMaxQ = 10;
 void gq_w_points_fx(gq_geom *g, const EvalView &E, const double2 *M, double *pot);
 void gq_w_centres_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *Q);
 void gq_w_fx_prepare(int dev);     // its tables on device dev
+// M2M of all levels in fixed point (gq_m2m_fx.cu)
+void gq_m2m_fx(gq_geom *g, const EvalView &E, double2 *M);
+void gq_m2m_fx_prepare(int dev);   // its table on device dev

@@ -233,10 +233,17 @@ __global__ void __launch_bounds__(128) k_l2l_t(EvalView E, int lstart, int lend,
     int q = (E.bix[c] & 1) | ((E.biy[c] & 1) << 1);
     const double2 *B = sB + bl * P1;
     const double2 *Uq = U + ((size_t)q * kTN + m) * kTN;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int k = m; k <= E.P; ++k) acc = cfma(__ldg(&Uq[k]), B[k], acc);
+    // four sums at a time: the products of one would wait for one another (64 cycles each)
+    double2 acc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = make_double2(0.0, 0.0);
+    int k = m;
+    for (; k + 3 <= E.P; k += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j] = cfma(__ldg(&Uq[k + j]), B[k + j], acc[j]);
+    for (; k <= E.P; ++k) acc[0] = cfma(__ldg(&Uq[k]), B[k], acc[0]);
     double2 *dst = L + (size_t)c * P1 + m;
-    *dst = cadd(*dst, acc);
+    *dst = cadd(*dst, cadd(cadd(acc[0], acc[1]), cadd(acc[2], acc[3])));
 }
 
 // ------------------------------------------------------------------ Stage 4: M2L over List 2
@@ -1866,6 +1873,7 @@ static const ConstTables &const_tables(int dev) {
     gq_dfl_log_table_host(&DT);
     gq_m2l_fx_prepare(dev);
     gq_w_fx_prepare(dev);
+    gq_m2m_fx_prepare(dev);
     ConstTables C;
     C.logt = upload_const((const double *)&LT, kGqLogN);
     FxLogTable FT;
@@ -1993,7 +2001,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // small problem are a chain of short kernels that leave most SMs idle.  Their
     // stream has the higher priority, so that the direct part, started first, does
     // not hold the chain up.  Both in order -> side by side: one curve 0.57 ->
-    // TIMEOV1 ms, 15 x 61-panel... TIMEOV2, 1.05 M nodes TIMEOV3.
+    // 0.43 ms, 35 ragged curves 2.15 -> 1.89, 1.05 M nodes 11.4 -> 10.3.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     GQ_CUDA(cudaStreamIsCapturing(st, &cap));
     const cudaStream_t sf = fmm_only ? st : g->s2;
@@ -2187,15 +2195,13 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                       128, 0, E, g->n_leaf_src, (const int *)g->leaf_src_boxes, g->M.p);
         }
     }
-    for (int l = g->nlev - 2; l >= 0; --l) {
-        int s = g->level_start_h[l], e = g->level_start_h[l + 1];
-        if (m2l_split)
+    if (m2l_split)
+        for (int l = g->nlev - 2; l >= 0; --l) {
+            const int s = g->level_start_h[l], e = g->level_start_h[l + 1];
             GQ_LAUNCH(ctx, k_m2m_split, gq_blocks((long long)(e - s) * P1, 128), 128, 0, E, s, e, T.tm2m2, g->M2.p);
-        else if (g->m2m_level_start_h[l + 1] > g->m2m_level_start_h[l])
-            GQ_LAUNCH(ctx, k_m2m_t, gq_blocks(g->m2m_level_start_h[l + 1] - g->m2m_level_start_h[l], 128 / P1),
-                      (128 / P1) * P1, 0, E, (const int *)g->m2m_boxes, g->m2m_level_start_h[l],
-                      g->m2m_level_start_h[l + 1], (const double2 *)T.tm2m, g->M.p);
-    }
+        }
+    else
+        gq_m2m_fx(g, E, g->M.p);
     mark(S_M2M, sf);
     if (m2l_split)
         GQ_LAUNCH(ctx, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
