@@ -241,6 +241,89 @@ __global__ void k_rs_scatter(const K *__restrict__ keys, const int *__restrict__
     }
 }
 
+// All passes of a short sort in one block: the passes of the kernels above are
+// three launches and a memset each, 27 us a pass whatever n.  A warp takes a
+// contiguous part of the elements, counts its digits, and after a scan over
+// (digit, warp) scatters them in order, so the sort is stable as the other is.  A
+// lane keeps its elements of a pass in registers, so that their loads overlap
+// (reading them twice from memory made 12,800 keys as slow as the launches).
+// 12,800 64-bit keys, 8 passes: 0.22 -> 0.18 ms; 6,000: build of one curve 1.70 -> 1.55 ms.
+constexpr int kRsSmallThreads = 1024;
+constexpr int kRsSmallItems = 14;
+constexpr int kRsSmall = kRsSmallThreads * kRsSmallItems;
+
+template <class K>
+__global__ void __launch_bounds__(kRsSmallThreads) k_rs_small(K *keys, int *vals, K *keys2, int *vals2, int n, int passes) {
+    constexpr int W = kRsSmallThreads / 32;
+    __shared__ int run[W][kRsDigits];
+    __shared__ int wtot[kRsDigits / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int per = ((n + W - 1) / W + 31) & ~31, i0 = min(n, w * per), i1 = min(n, i0 + per);   // per <= 32 items
+    const unsigned lt = (1u << lane) - 1u;
+    for (int ps = 0; ps < passes; ++ps) {
+        const int shift = ps * kRsBits;
+        K *ka = ps & 1 ? keys2 : keys, *kb = ps & 1 ? keys : keys2;
+        int *va = ps & 1 ? vals2 : vals, *vb = ps & 1 ? vals : vals2;
+        K k[kRsSmallItems];
+        int v[kRsSmallItems];
+#pragma unroll
+        for (int c = 0; c < kRsSmallItems; ++c) {
+            const int i = i0 + 32 * c + lane;
+            k[c] = i < i1 ? ka[i] : 0;
+            v[c] = i < i1 ? va[i] : 0;
+        }
+        for (int i = lane; i < kRsDigits; i += 32) run[w][i] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < kRsSmallItems; ++c)
+            if (i0 + 32 * c + lane < i1) atomicAdd(&run[w][(int)((k[c] >> shift) & (kRsDigits - 1))], 1);
+        __syncthreads();
+        // exclusive prefix over (digit, warp): a thread per digit
+        int tot = 0;
+        if (threadIdx.x < kRsDigits)
+            for (int j = 0; j < W; ++j) {
+                const int c = run[j][threadIdx.x];
+                run[j][threadIdx.x] = tot;
+                tot += c;
+            }
+        int x = tot;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (threadIdx.x < kRsDigits && lane == 31) wtot[w] = x;
+        __syncthreads();
+        if (threadIdx.x < kRsDigits) {
+            int base = x - tot;
+            for (int j = 0; j < w; ++j) base += wtot[j];
+            for (int j = 0; j < W; ++j) run[j][threadIdx.x] += base;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < kRsSmallItems; ++c) {
+            if (i0 + 32 * c >= i1) break;
+            const bool valid = i0 + 32 * c + lane < i1;
+            const int d = valid ? (int)((k[c] >> shift) & (kRsDigits - 1)) : kRsDigits;
+            const unsigned m = __match_any_sync(0xffffffffu, d);
+            const int at = valid ? run[w][d] : 0;
+            __syncwarp();
+            if (valid) {
+                const int pos = at + __popc(m & lt);
+                kb[pos] = k[c];
+                vb[pos] = v[c];
+                if (lane == __ffs(m) - 1) run[w][d] = at + __popc(m);
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+    }
+    if (passes & 1)
+        for (int i = threadIdx.x; i < n; i += kRsSmallThreads) {
+            keys[i] = keys2[i];
+            vals[i] = vals2[i];
+        }
+}
+
 template <class K>
 void radix_sort_impl(gq_ctx *ctx, K *keys, int *vals, long long n, int bits) {
     if (n <= 1 || bits <= 0) return;
@@ -249,6 +332,11 @@ void radix_sort_impl(gq_ctx *ctx, K *keys, int *vals, long long n, int bits) {
     dbuf<int> v2, hist, offs, tmp;
     k2.alloc(n);
     v2.alloc(n);
+    if (n <= kRsSmall) {
+        GQ_LAUNCH(ctx, k_rs_small<K>, 1, kRsSmallThreads, 0, keys, vals, k2.p, v2.p, (int)n, (bits + kRsBits - 1) / kRsBits);
+        GQ_CUDA(cudaStreamSynchronize(ctx->stream));   // the temporaries are freed on return
+        return;
+    }
     long long nh = (long long)kRsDigits * nblk;
     hist.alloc(nh);
     offs.alloc(nh + 1);

@@ -192,3 +192,26 @@ def test_list3_far_in_fixed_point(p, q):
         # inside-disk sources of these coarse panels amplify the direct sums' rounding by |r/w|^q
         assert (a - b).abs().max().item() <= 1e-13 * b.abs().max().item() * 4.0 ** max(0, q - 5), kern
     geo.close()
+
+
+@pytest.mark.parametrize("panels", [24, 28, 29])
+def test_build_around_the_one_block_sort(panels):
+    """Particle counts below, at and above the 14,336 of the one-block sort (64
+    sources and 32 centres a panel and 10,240 point targets, some of which the
+    centres take): the same keys have to come out in the same stable order, so the
+    tree and owners equal the oracle's."""
+    import oracle
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_04070_gb300 import Geometry, params_default
+    g = workloads.small_grid(1, 1, panels, 14336 - 96 * 28, seed=2)
+    geo = Geometry(g, params_default(p_qbx=5, p_fmm=10, n_max=32))
+    geo.build()
+    o = oracle.Oracle(g, oracle.default_params(g))
+    for a, b in zip(geo.owners(), o.owners()):
+        assert np.array_equal(a, b)
+    bx, bo = geo.boxes(), o.boxes()
+    for k in ("level", "ix", "iy", "parent", "nsrc", "nctr", "ntgt"):
+        assert np.array_equal(bx[k], bo[k]), k
+    geo.close()
