@@ -20,6 +20,7 @@
 //   L2L  beta_m  = sum_{k>=m} C(k,m) b_k y^(k-m)                             (eq. l2l)
 // M2L is evaluated in that factored form: scale a_k by y^-k, apply the real
 // matrix C(m+k-1,k-1) shared by every pair, scale by (-1)^m y^-m.
+#include <exception>
 #include <math.h>
 #include <stdlib.h>
 
@@ -2160,11 +2161,19 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     };
 
     // ---- FMM passes: the context's launches go to their stream until the join
+    // (an exception waits for them: the geometry's buffers are then unused)
     struct OnStream {
         gq_ctx *c;
-        cudaStream_t own;
-        OnStream(gq_ctx *c_, cudaStream_t s_) : c(c_), own(c_->stream) { c->stream = s_; }
-        ~OnStream() { c->stream = own; }
+        cudaStream_t own, s;
+        int depth = std::uncaught_exceptions();
+        OnStream(gq_ctx *c_, cudaStream_t s_) : c(c_), own(c_->stream), s(s_) { c->stream = s_; }
+        ~OnStream() {
+            c->stream = own;
+            if (std::uncaught_exceptions() > depth) {
+                cudaStreamSynchronize(s);
+                cudaGetLastError();
+            }
+        }
     };
     {
     OnStream passes(ctx, sf);
