@@ -194,21 +194,27 @@ def test_list3_far_in_fixed_point(p, q):
     geo.close()
 
 
-@pytest.mark.parametrize("panels", [24, 28, 29])
-def test_build_around_the_one_block_sort(panels):
-    """Particle counts below, at and above the 14,336 of the one-block sort (64
-    sources and 32 centres a panel and 10,240 point targets, some of which the
-    centres take): the same keys have to come out in the same stable order, so the
-    tree and owners equal the oracle's."""
+@pytest.mark.parametrize("n", [12289, 14335, 14336, 14337])
+def test_build_around_the_one_block_sort(n):
+    """Particle counts (sources, centres and point targets) far below, just below,
+    at and just above the 14,336 of the one-block sort: the same keys have to come
+    out in the same stable order, so the tree and owners equal the oracle's."""
     import oracle
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_1801_04070_gb300 import Geometry, params_default
-    g = workloads.small_grid(1, 1, panels, 14336 - 96 * 28, seed=2)
+    g = workloads.small_grid(1, 1, 128, 20000, seed=2)
+    kind, _ = oracle.Oracle(g, oracle.default_params(g)).association()
+    base = len(g["up_xy"]) + 2 * len(g["base_xy"])             # 12,288
+    points = np.cumsum(kind[:20000] == 0)                      # targets no centre takes
+    keep = int(np.searchsorted(points, n - base)) + 1          # the shortest prefix with n - base points
+    g["tgt_xy"] = np.ascontiguousarray(g["tgt_xy"][:keep])
+    g["tgt_onsurf"] = np.ascontiguousarray(g["tgt_onsurf"][:keep])
     geo = Geometry(g, params_default(p_qbx=5, p_fmm=10, n_max=32))
     geo.build()
     o = oracle.Oracle(g, oracle.default_params(g))
+    assert base + o.npt == n
     for a, b in zip(geo.owners(), o.owners()):
         assert np.array_equal(a, b)
     bx, bo = geo.boxes(), o.boxes()
