@@ -1544,8 +1544,7 @@ void dispatch_near_centres_f32(gq_ctx *ctx, const EvalView &E, const MixedView &
 // its reciprocal, log|w|, r/w) and the powers (r/w)^m are formed once and
 // serve ND densities, each of which adds only its strength times the power.
 // strm: ND strength arrays of the sorted sources, sstride apart; Qm: ND
-// coefficient arrays [nc][q+1], qstride apart.  Same layout and sums as
-// k_near_centres otherwise.
+// coefficient arrays [nc][q+1], qstride apart.
 template <int QQ, int KERNEL, int ND>
 __device__ void near_centres_multi_box(const EvalView &E, int b, const double2 *__restrict__ strm, long long sstride,
                                        double2 *__restrict__ Qm, long long qstride, NearRanges &R, int *wsum,
@@ -2118,7 +2117,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             auto ks = k_near_points_f32<GQ_S>;
             GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, X, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
-        } else if (split) {   // pairs: 0.72 ms where fixed point takes 1.11 (0.86 M targets)
+        } else if (split) {   // pairs: 0.72 ms where fixed point takes 0.78 (0.86 M targets)
             auto kd = k_near_points_split<GQ_D>;
             auto ks = k_near_points_split<GQ_S>;
             GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, SX, g->n_pt_boxes,

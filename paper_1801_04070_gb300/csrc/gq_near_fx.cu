@@ -342,12 +342,13 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
 
 // Potential at the point targets for S, sum q log|t - y| (coincident sources
 // skipped): a block per target box, a warp per target, lanes stride over the
-// staged sources; |w|^2 in FP64 (four instructions of the 12.7 that the FP64 form
-// took a pair, which bound it), logarithm, products and sums in fixed point.  What
-// bounds it now is the latency of a box's short work (about ten targets and 70
-// sources): resident blocks over several boxes 1.3 ms, without staging 1.5, a warp a
-// box 1.8, a warp per eight targets 1.6.  0.86 M point targets: 1.37 -> 1.11 ms, 0.20 M:
-// 0.53 -> 0.37.
+// staged sources; |w|^2 in FP64, logarithm, products and sums in fixed point.  The
+// FP64 pipe bounds it (83 % busy with 11.6 instructions a pair of a warp, at ten
+// targets and 70 sources a box): four a pair are |w|^2, so the conversions of
+// a target's sum wait in the lanes until 32 targets are converted by one
+// instruction, and the strengths' sum is formed once a tile.  Resident
+// blocks over several boxes, no staging, a warp a box or several targets a warp
+// were slower.  0.86 M point targets: 1.37 (FP64) -> 1.11 -> 0.78 ms.
 __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, const int *__restrict__ work,
                                                                  double *__restrict__ pot) {
     __shared__ NearRanges R;
@@ -376,6 +377,19 @@ __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, con
             const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
             if (v0) __syncthreads();
             const int qe = fx_stage<GQ_S>(E, R, v0, v1, sy, sq, ssum, smax);
+            const double sc = pow2_clamped(qe + 1 - 55);
+            const double q0 = qe > 0 ? fx_strength_sum(ssum) * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264) : 0.0;
+            // the sums of up to 32 targets wait in the lanes and are converted together
+            long long khi = 0;
+            int klo = 0, kt = -1, held = 0;
+            auto flush = [&]() {
+                if (kt >= 0) {
+                    const double x = fma((double)khi, 16777216.0, (double)klo) * sc + q0;
+                    pot[kt] = first ? x : pot[kt] + x;
+                    kt = -1;
+                }
+                held = 0;
+            };
             for (int t = tb + w; t < te; t += kFxWarps) {
                 const double2 tz = E.sp_xy[t];
                 long long acc = 0;
@@ -393,18 +407,20 @@ __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, con
                 nmin = __reduce_min_sync(0xffffffffu, nmin);
                 nmax = __reduce_max_sync(0xffffffffu, nmax);
                 const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20);
-                double x;
                 if (qe > 0 && (n == 0 || (emin >= 128 && emax <= 1920 && emax - eref <= 40 && eref - emin <= 40))) {
                     // 12 terms below 2^58.8 a lane: the sum over lanes in two words
                     int lo = (int)(acc & ((1 << 24) - 1));
                     long long hi = acc >> 24;
                     for (int o = 16; o > 0; o >>= 1) hi += __shfl_xor_sync(0xffffffffu, hi, o);
                     lo = __reduce_add_sync(0xffffffffu, lo);
-                    const double sc = pow2_clamped(qe + 1 - 55);
-                    x = fma((double)hi, 16777216.0, (double)lo) * sc +
-                        fx_strength_sum(ssum) * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264);
+                    if (lane == held) {
+                        khi = hi;
+                        klo = lo;
+                        kt = t;
+                    }
+                    if (++held == 32) flush();
                 } else {   // in FP64, infinities and coincident sources included
-                    x = 0.0;
+                    double x = 0.0;
                     int r = 0;
                     for (int v = v0 + lane; v < v1; v += 32) {
                         while (R.pre[r + 1] <= v) ++r;
@@ -414,9 +430,10 @@ __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, con
                         x = fma(E.str[s].x, n2 == 0.0 ? 0.0 : gq_log_half(n2, E.logt), x);
                     }
                     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                    if (lane == 0) pot[t] = first ? x : pot[t] + x;
                 }
-                if (lane == 0) pot[t] = first ? x : pot[t] + x;
             }
+            flush();
             first = false;
         }
     }

@@ -221,3 +221,31 @@ def test_build_around_the_one_block_sort(n):
     for k in ("level", "ix", "iy", "parent", "nsrc", "nctr", "ntgt"):
         assert np.array_equal(bx[k], bo[k]), k
     geo.close()
+
+
+@pytest.mark.parametrize("n", [1, 124, 125, 128, 129, 260, 700])
+def test_many_point_targets_in_a_box(n):
+    """Point targets of one leaf around the counts at which the four warps of
+    k_near_points_fx convert the 32 sums they hold (125 .. 128: the first full
+    warp), over two tiles of sources; against long double sums.  The bound is
+    64 units of 2^-53 of the terms' absolute sum (logarithm 2 units, products and
+    sums below one, conversion and potential's factor 3; 512 terms at random)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_04070_gb300 import Geometry, params_default
+    g = workloads.small_grid(1, 1, 8, 0, seed=4)
+    rng = np.random.default_rng(n)
+    g["tgt_xy"] = np.stack([rng.uniform(-6, 6, n), rng.uniform(3, 6, n)], 1)   # outside every centre's disk
+    g["tgt_onsurf"] = np.full(n, -1, np.int32)
+    geo = Geometry(g, params_default(p_qbx=5, p_fmm=10, n_max=4000))
+    geo.build()
+    assert geo.npt == n and geo.info.nbox == 1
+    out = np.empty(n)
+    geo.eval("S", g["density"], out)
+    geo.close()
+    q = np.asarray(_strengths(g, g["density"]), np.longdouble)
+    d = g["tgt_xy"].astype(np.longdouble)[:, None, :] - g["up_xy"].astype(np.longdouble)[None, :, :]
+    terms = q[None, :] * np.log(np.hypot(d[..., 0], d[..., 1]))
+    ref = -terms.sum(1) / (2 * np.longdouble(np.pi))
+    assert np.all(np.abs(out - ref) <= 64 * 2.0 ** -53 * np.abs(terms).sum(1) / (2 * np.pi))
