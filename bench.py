@@ -192,13 +192,13 @@ def work_model(geo, p, q, kernel="S"):
     v_pairs = int(len(L["V"][1]))
     wf_ctr = int((wf * nctr).sum())
     return {
-        5: dict(name="k_near_centres", units=pairs_ctr, flops_per_unit=14 * q + 20, unit="(source, centre) pair"),
-        6: dict(name="k_near_points", units=pairs_pt, flops_per_unit=10 + (LOG_FLOPS if kernel == "S" else 0),
+        5: dict(name="k_near_centres_fx", units=pairs_ctr, flops_per_unit=14 * q + 20, unit="(source, centre) pair"),
+        6: dict(name="k_near_points_fx" if kernel == "S" else "k_near_points", units=pairs_pt, flops_per_unit=10 + (LOG_FLOPS if kernel == "S" else 0),
                 unit="(source, point) pair"),
-        2: dict(name="k_m2l_tc" if p <= 15 else "k_m2l", units=v_pairs, flops_per_unit=8 * (p + 1) ** 2,
+        2: dict(name="k_m2l_tc" if p <= 15 else "k_m2l_fx", units=v_pairs, flops_per_unit=8 * (p + 1) ** 2,
                 unit="List 2 pair (FP64-equivalent flops of the translation)"),
         7: dict(name="k_w_centres_tc" if (p <= 16 and q <= 15 and math.comb(q + p - 1, p - 1) < 1 << 24)
-                else "k_w_centres_q", units=wf_ctr, flops_per_unit=8 * (p + 1) * (q + 1),
+                else "k_w_centres_fx" if q <= 10 else "k_w_centres_q", units=wf_ctr, flops_per_unit=8 * (p + 1) * (q + 1),
                 unit="(List 3 far box, centre) pair (FP64-equivalent flops of the translation)"),
     }
 
@@ -648,19 +648,23 @@ def run_gpu(args, rank, world, local):
             if L.gq_probe_fma_peak(ctx, what, C.byref(v)) == 0:
                 others[name] = v.value
         per_kernel = {}
-        # FP64 instructions per unit measured by ncu (profiles/fp64_inst.json): the FP64 pipe
-        # issues one instruction per slot whatever its kind, at the measured FMA peak / 2
-        fi = os.path.join(ROOT, "profiles", "fp64_inst.json")
+        # the direct kernels work in 64-bit fixed point: instructions per unit on the pipe that
+        # takes the 32 x 32 bit multiply-adds (half of the FP32 lanes), counted by ncu
+        # (profiles/int_inst.json), against its issue rate, a quarter of the measured FP32
+        # FMA flops (a multiply-add with a 64-bit result takes two issue slots, so the
+        # pipe is busier than this says).  A fraction above 1 of "achieved" / "peak" below says that FP64 FMAs
+        # could not do this work in the time.
+        fi = os.path.join(ROOT, "profiles", "int_inst.json")
         inst = json.load(open(fi)) if os.path.exists(fi) else {}
         for i, mm in model.items():
             a = mm["units"] * mm["flops_per_unit"] / (stage_ms[i] * 1e-3) / 1e12
             per_kernel[mm["name"]] = {"achieved": a, "frac": a / peak.value, "ms_per_launch": float(stage_ms[i]),
                                       "units_per_launch": mm["units"], "flops_per_unit": mm["flops_per_unit"],
                                       "unit_of_work": mm["unit"]}
-            if args.kernel == "S" and mm["name"] in inst:
+            if args.kernel == "S" and mm["name"] in inst and others.get("fp32_fma"):
                 rate = mm["units"] * inst[mm["name"]] / (stage_ms[i] * 1e-3) / 1e12
-                per_kernel[mm["name"]]["fp64_inst_per_unit"] = inst[mm["name"]]
-                per_kernel[mm["name"]]["fp64_issue_frac"] = rate / (peak.value / 2)
+                per_kernel[mm["name"]]["int_pipe_inst_per_unit"] = inst[mm["name"]]
+                per_kernel[mm["name"]]["int_pipe_issue_frac"] = rate / (others["fp32_fma"] / 4)
         roof = {"bound": "alu", "kernel": m["name"], "achieved": achieved, "peak": peak.value,
                 "unit": "TFLOP/s", "frac": achieved / peak.value, "traffic": traffic,
                 "peak_source": peak_src, "units_per_launch": m["units"], "unit_of_work": m["unit"],

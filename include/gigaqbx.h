@@ -75,7 +75,13 @@ enum { GQ_S = 0, GQ_D = 1, GQ_SP = 2 };
  *                 reports up to 20% slack as harmless); otherwise it is an
  *                 ordinary FMM point target.
  *  eps          : requested accuracy (used for orders of 0 and by the mixed modes).
- *  precision    : GQ_PREC_FP64 (default): every stage in FP64.
+ *  precision    : GQ_PREC_FP64 (default): every stage to FP64 accuracy.  The
+ *                 direct sums to the centres (and of S to the point
+ *                 targets), the translations of List 2 with p_fmm >= 16,
+ *                 those of List 3 far that the tensor cores do not take, and
+ *                 M2M run in 64-bit fixed point on the integer pipes (58 to
+ *                 62 fraction bits, inputs and sums at shared exponents),
+ *                 the rest in FP64 or as stated at m2l.
  *                 GQ_PREC_MIXED: a tier chosen from eps.
  *                 eps >= 5e-6: the direct interactions (Lists 1, 3 close,
  *                 4 close to centres and to point targets) and the List 3
@@ -85,11 +91,13 @@ enum { GQ_S = 0, GQ_D = 1, GQ_SP = 2 };
  *                 the larger for D; below eps/5).
  *                 1e-12 <= eps < 5e-6: the same steps run in double-FP32
  *                 pairs (about 48 significant bits; measured 1e-15 .. 2e-13
- *                 relative to the FP64 path).  In both tiers a source inside
- *                 a centre's expansion disk (|r/w| > 1, where rounding would
- *                 grow as |r/w|^m) is taken in FP64, below eps = 1e-10 also
- *                 a source within 1/8 of the box half-width of a point
- *                 target; the List 3 far
+ *                 relative to the FP64 path), but for the direct sums to
+ *                 the centres, which are those of the FP64 mode (fixed point
+ *                 is faster than pairs there).  In the first tier a source
+ *                 inside a centre's expansion disk (|r/w| > 1, where rounding
+ *                 would grow as |r/w|^m) is taken in FP64, in the second,
+ *                 below eps = 1e-10, a source within 1/8 of the box
+ *                 half-width of a point target; the List 3 far
  *                 translation to centres (M2QBXL) runs in pairs when the tree
  *                 has at most 24 levels.  The translations M2M, M2L, L2L,
  *                 L2QBXL, the P2M and P2L sums, L2P and the final QBX
@@ -130,8 +138,10 @@ enum { GQ_PREC_FP64 = 0, GQ_PREC_MIXED = 1, GQ_PREC_MIXED_FMM = 2 };
  *       p_fmm - 1) < 2^24: the binomial sums of each (centre, box) pair as a
  *       product of 64-bit fixed-point pair entries (eight 8-bit digits) and
  *       the constant binomial matrix (three 8-bit digits);
- *     otherwise FP64 FMAs.
- *   GQ_M2L_FP64: always the FP64 FMA kernels. */
+ *     otherwise as with GQ_M2L_FP64.
+ *   GQ_M2L_FP64: never on the tensor cores: List 2 by FP64 FMAs for p_fmm <= 15
+ *       and in 64-bit fixed point above; List 3 far to the centres in fixed
+ *       point for p_qbx <= 10, by FP64 FMAs above. */
 enum { GQ_M2L_AUTO = 0, GQ_M2L_FP64 = 1 };
 
 /* level_restrict = 1: a level-restricted tree (Sec. 4.6, remark on
@@ -184,7 +194,9 @@ typedef struct {
                                  4 L2L, 5 direct to centres (Lists 1, 3 close, 4 close),
                                  6 direct to point targets, 7 List 3 far to centres,
                                  8 List 3 far to point targets, 9 L2QBXL + L2P,
-                                 10 final QBX evaluation, 11 unused */
+                                 10 final QBX evaluation, 11 unused.  5 and 6 run on the
+                                 context's stream beside the others: the times of the
+                                 two sides overlap */
 } gq_stats;
 
 /* Tree and list sizes after gq_build. */
@@ -289,12 +301,11 @@ gq_status gq_gmres(gq_geom *g, const double *rhs, double tol, int maxit, int res
  * 4, 8 and 16 streams, times replays and keeps the fastest (cached per batch
  * shape; written to the file named by GQ_AUTOTUNE_CACHE if set); later calls
  * with the same arguments only replay the graph.  The geometries must stay
- * alive and must not be rebuilt while the batch exists.  In FP64 mode the
- * direct part of the QBX coefficients is formed for up to four densities of a
- * geometry at a time (the per-pair geometry and the powers (r/w)^m shared),
- * which rounds differently from one gq_eval per density: results agree with
- * gq_eval to about 1e-14 relative and repeat bit for bit from call to call;
- * the rest of the evaluation uses the gq_eval kernels. */
+ * alive and must not be rebuilt while the batch exists.  A branch runs the kernels of
+ * gq_eval, its densities one after another; only the persistent launch of
+ * gq_batch_mode 0 forms the direct part for several densities at a time, in
+ * FP64, and so agrees with gq_eval to about 1e-14 relative.  Either way the
+ * results repeat bit for bit from call to call. */
 typedef struct gq_batch gq_batch;
 gq_status gq_batch_create(gq_ctx *ctx, int ngeom, gq_geom *const *geoms, gq_batch **out);
 gq_status gq_batch_destroy(gq_batch *b);
@@ -320,8 +331,8 @@ gq_status gq_batch_streams(const gq_batch *b, int *streams);
  *     wait status.  Other configurations use the branches of mode 1.
  *   mode 1: every evaluation in the per-geometry branches (as described at
  *     gq_batch_eval).
- * The results equal those of mode 1 to rounding of the final sums (the same
- * kernels' arithmetic). */
+ * The results equal those of mode 1 to rounding of the direct and final sums
+ * (the direct sums of mode 1 run in 64-bit fixed point). */
 gq_status gq_batch_mode(gq_batch *b, int mode);
 /* Target boxes per direct item of the persistent launch in use (0: the
  * captured graph does not use the persistent launch). */
@@ -424,7 +435,8 @@ gq_status gq_set_orders(gq_geom *g, int p_qbx, int p_fmm);
  * (GQ_ERR_STATE otherwise).  The first call on a device sets the array up
  * (looks up its device address, writes the tables and waits for the copies
  * with a device synchronisation); make that first call before any stream
- * capture.  The kernels are those of gq_eval in FP64 mode.
+ * capture.  Its kernels work in FP64, but for the direct sums to the centres,
+ * which are those of gq_eval; results agree with gq_eval to rounding.
  * All calls share the one array and it keeps the last call's contents, so
  * calls whose device work overlaps (different streams or contexts) race;
  * order them on one stream.  No memory is allocated or freed by this call. */
