@@ -13,8 +13,11 @@
 // Formats (bits behind the binary point in brackets): u = r/w [62], t_m = q u^m
 // [60] with the strengths scaled to at most 1/2, products rounded at 2^-60.
 // |u| <= 1 when no source is inside the centre's disk; the loop records the
-// smallest |w|^2, and a centre that meets |u| > 1 + 1/64 is summed again with
-// the smallest |w| as its radius (the sums are then scaled by (r/|w|)^m).
+// smallest |w|^2, and a centre that meets |u| > 1 + 1/64 is summed again.  While
+// (r/|w|)^q <= 2^4 (centres on the inner side of a sharp bend) that is with the
+// smallest |w| as its radius, and the sums are then scaled by (r/|w|)^m; above, the
+// sources inside are left out and their powers summed in FP64, since a scale that
+// holds them would leave the other sources' terms few bits or none.
 // Sums: 12 terms a lane (tiles of 384 sources), |t_m| < 0.65, stay below 2^63;
 // the warp's sum is taken at 2^-60 (2^-55 if the lanes' sums are that large).  Error against long double sums on the nodes
 // of a starfish grid (272 sources, q = 8, root mean square, in units of the
@@ -23,9 +26,11 @@
 //
 // The scale is that of the tile's own strengths, so that a strong source far away
 // costs a centre no accuracy.  Strengths that have none (infinite, NaN, exponents
-// near the ends of the range) and sources at the centre itself go through near_centre_slow, an
-// FP64 sum order by order with the arithmetic's own infinities and NaN.
+// near the ends of the range) go through near_centre_fp64 whole, with the arithmetic's
+// own infinities and NaN.
 #include <math.h>
+
+#include <type_traits>
 
 #include "gq_eval.cuh"
 #include "gq_math.cuh"
@@ -74,38 +79,60 @@ constexpr RsPlace rs_place(int n, int i) {
     return RsPlace{lane, i};
 }
 
-// The sources [v0, v1) of the loaded ranges in FP64, order by order (every warp
-// lane takes part): any strength or distance, infinities and NaN included.
+// In FP64: the sources [v0, v1) of the loaded ranges (every warp lane takes part; with
+// infinities and NaN), or the powers (no logarithms) of those whose |w|^2 has an upper
+// word below nlim, added to dst (first: written).  Nine orders a sweep: their sums fit
+// the registers.
+constexpr unsigned kAllSources = 0xffffffffu;
 template <int KERNEL>
-__device__ __noinline__ void near_centre_slow(const EvalView &E, const NearRanges &R, int v0, int v1, double2 cz, double rc,
-                                              int QQ, int qc, double2 *dst, bool first) {
+__device__ __noinline__ void near_centre_fp64(const EvalView &E, const NearRanges &R, int v0, int v1, double2 cz, double rc,
+                                              int QQ, int qc, unsigned nlim, double2 *dst, bool first) {
+    constexpr int NC = 9;
     const int lane = threadIdx.x & 31;
-    for (int m = 0; m <= QQ; ++m) {
-        double2 acc = make_double2(0.0, 0.0);
-        int r = 0;
-        if (m <= qc)
-            for (int v = v0 + lane; v < v1; v += 32) {
+    for (int m0 = 0; m0 <= QQ; m0 += NC) {
+        double2 acc[NC];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) acc[i] = make_double2(0.0, 0.0);
+        if (m0 <= qc)
+            for (int v = v0 + lane, r = 0; v < v1; v += 32) {
                 while (R.pre[r + 1] <= v) ++r;
                 const int s = R.beg[r] + (v - R.pre[r]);
-                const double2 y = E.s_xy[s], st = E.str[s];
-                const double wx = y.x - cz.x, wy = y.y - cz.y, n2 = wx * wx + wy * wy;
-                if (KERNEL != GQ_D && m == 0) {
-                    // a coincident source has log term 0
-                    acc.x = fma(st.x, n2 == 0.0 ? 0.0 : gq_log_half(n2, E.logt), acc.x);
-                    continue;
-                }
+                const double2 y = E.s_xy[s];
+                const double wx = y.x - cz.x, wy = y.y - cz.y, n2 = fma(wx, wx, wy * wy);
+                if ((unsigned)(fx_bits(n2) >> 32) >= nlim) continue;
+                const double2 st = E.str[s];
                 const double inv = gq_rcp(n2);
                 const double2 winv = make_double2(wx * inv, -wy * inv);
                 const double2 u = make_double2(rc * winv.x, rc * winv.y);
-                double2 t = KERNEL == GQ_D ? cmul(st, winv) : make_double2(st.x * u.x, st.x * u.y);
-                for (int i = KERNEL == GQ_D ? 0 : 1; i < m; ++i) t = cmul(t, u);
-                acc = cadd(acc, t);
+                double2 t = KERNEL == GQ_D ? cmul(st, winv) : make_double2(st.x * u.x, st.x * u.y);   // order 0 (D) or 1
+                if (m0) {
+                    double2 p = u;
+                    for (int i = 0; i < 3; ++i) p = cmul(p, p);
+                    t = cmul(t, p);
+                    if (KERNEL == GQ_D) t = cmul(t, u);
+                } else if (KERNEL != GQ_D && nlim == kAllSources) {
+                    // a coincident source has log term 0
+                    acc[0].x = fma(st.x, n2 == 0.0 ? 0.0 : gq_log_half(n2, E.logt), acc[0].x);
+                }
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    if (KERNEL != GQ_D && i == 0 && m0 == 0) continue;
+                    acc[i] = cadd(acc[i], t);
+                    t = cmul(t, u);
+                }
             }
-        for (int o = 16; o > 0; o >>= 1)
-            acc = cadd(acc, make_double2(__shfl_xor_sync(0xffffffffu, acc.x, o), __shfl_xor_sync(0xffffffffu, acc.y, o)));
-        if (lane == 0) {
-            if (KERNEL != GQ_D && m >= 1) acc = cscale(acc, c_ninv[m]);
-            dst[m] = first ? acc : cadd(dst[m], acc);
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            const int m = m0 + i;
+            if (m > QQ) break;
+            for (int o = 16; o > 0; o >>= 1)
+                acc[i] = cadd(acc[i], make_double2(__shfl_xor_sync(0xffffffffu, acc[i].x, o),
+                                                   __shfl_xor_sync(0xffffffffu, acc[i].y, o)));
+            if (lane == 0) {
+                double2 x = m <= qc ? acc[i] : make_double2(0.0, 0.0);
+                if (KERNEL != GQ_D && m >= 1) x = cscale(x, c_ninv[m]);
+                dst[m] = first ? x : cadd(dst[m], x);
+            }
         }
     }
 }
@@ -222,26 +249,33 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                 const double rc = E.sc_r[c];
                 const int qc = E.qc ? E.qc[c] : QQ;
                 double2 *dst = Qout + (size_t)c * (QQ + 1);
-                double re = rc;
+                double re = rc;      // u = re/w
                 bool slow = !scaled;
+                unsigned nlim = 0;   // terms of sources with an upper word of |w|^2 below it are formed in FP64
                 long long acc[NV];   // S: 0 the log sum, 1 unused, then Re, Im of each order; D: Re, Im of each order
-                for (int pass = 0; !slow; ++pass) {
+                unsigned nmin = 0xffffffffu, nmax = 0;   // upper words of |w|^2
+                auto sweep = [&](auto without) {
                     const uint64_t rb = fx_bits(re);
                     const gfx Rm = fx_bal((long long)(fx_mant(rb) << 9));
                     const int er = fx_expo(rb);
+                    nmin = 0xffffffffu;
+                    nmax = 0;
 #pragma unroll
                     for (int i = 0; i < NV; ++i) acc[i] = 0;
-                    unsigned nmin = 0xffffffffu, nmax = 0;   // upper words of |w|^2
                     for (int v = lane; v < n; v += 32) {
                         const double2 y = sy[v];
                         const double wx = y.x - cz.x, wy = y.y - cz.y;
                         const double n2 = fma(wx, wx, wy * wy);
                         const uint64_t nb = fx_bits(n2);
-                        nmin = min(nmin, (unsigned)(nb >> 32));
+                        str_t sv = sq[v];
+                        if constexpr (KERNEL != GQ_D)
+                            acc[0] += fx_mul(gfx{sv.x, sv.y}, fx_bal(fx_log_half(nb, eref, shl_, stj)));
+                        const bool in = without.value && (unsigned)(nb >> 32) < nlim;
+                        if (in) sv = str_t{};
+                        if (!in || KERNEL != GQ_D) nmin = min(nmin, (unsigned)(nb >> 32));
                         nmax = max(nmax, (unsigned)(nb >> 32));
                         gfx ux, uy, nuy;
                         fx_ratio(wx, wy, nb, Rm, er, ux, uy, nuy);
-                        const str_t sv = sq[v];
                         long long tr, ti;
                         if constexpr (KERNEL == GQ_D) {
                             fx_cmul30(gfx30{sv.x, sv.y}, gfx30{sv.z, sv.w}, ux, uy, nuy, tr, ti);
@@ -249,7 +283,6 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                             acc[1] += ti;
                         } else {
                             const gfx a{sv.x, sv.y};
-                            acc[0] += fx_mul(a, fx_bal(fx_log_half(nb, eref, shl_, stj)));
                             tr = fx_mul(a, ux);
                             ti = fx_mul(a, uy);
                             acc[2] += tr;
@@ -268,21 +301,28 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                     }
                     nmin = __reduce_min_sync(0xffffffffu, nmin);
                     nmax = __reduce_max_sync(0xffffffffu, nmax);
-                    if (n == 0) break;
-                    // |w|^2 a normal number far from the range's ends, the logarithms below 14
-                    const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20);
-                    if (emin < 128 || emax > 1920 || er < 128 || er > 1920 ||
-                        (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40))) {
-                        slow = true;
+                };
+                if (!slow) {
+                    for (;;) {
+                        sweep(std::false_type{});
+                        // a source inside the disk, |u|^2 > 1 + 1/32
+                        const double wmin2 = __hiloint2double((int)nmin, 0);
+                        if (n == 0 || re != rc || !(rc * rc > wmin2 * (1.0 + 1.0 / 32))) break;
+                        if (rc * rc * exp2f(-8.0f / qc) <= wmin2) {
+                            re = sqrt(wmin2);
+                            continue;
+                        }
+                        nlim = (unsigned)(fx_bits(rc * rc * (32.0 / 33)) >> 32) + 1;
+                        sweep(std::true_type{});
                         break;
                     }
-                    // a source inside the disk: |u|^2 > 1 + 1/32
-                    const double wmin2 = __hiloint2double((int)nmin, 0);
-                    if (pass > 0 || re * re <= wmin2 * (1.0 + 1.0 / 32)) break;
-                    re = sqrt(wmin2);
+                    // |w|^2 a normal number far from the range's ends, the logarithms below 14
+                    const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20), er = fx_expo(fx_bits(re));
+                    slow = n > 0 && (emin < 128 || emax > 1920 || er < 128 || er > 1920 ||
+                                     (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40)));
                 }
                 if (slow) {
-                    near_centre_slow<KERNEL>(E, R, v0, v1, cz, rc, QQ, qc, dst, first);
+                    near_centre_fp64<KERNEL>(E, R, v0, v1, cz, rc, QQ, qc, kAllSources, dst, first);
                     continue;
                 }
                 // exact sum of the log terms as two words; the others at 2^-60 or as close to
@@ -334,6 +374,10 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                         }
                         d[i] = first ? x : d[i] + x;
                     }
+                if (nlim) {
+                    __syncwarp();   // lane 0 adds to what the lanes have written
+                    near_centre_fp64<KERNEL>(E, R, v0, v1, cz, rc, QQ, qc, nlim, dst, false);
+                }
             }
             first = false;
         }
