@@ -24,10 +24,10 @@
 // strength scale), FP64 form -> this: Q_0 2^-46.3 -> 2^-50.9, Q_1 2^-48.7 ->
 // 2^-53.0, Q_4 2^-50.9 -> 2^-52.1, Q_8 2^-50.5 -> 2^-51.5.
 //
-// The scale is that of the tile's own strengths, so that a strong source far away
-// costs a centre no accuracy.  Strengths that have none (infinite, NaN, exponents
-// near the ends of the range) go through near_centre_fp64 whole, with the arithmetic's
-// own infinities and NaN.
+// The scale is that of the tile's own strengths.  Strengths that have none (infinite,
+// NaN, exponents near the ends of the range) and centres whose terms are weak beside
+// it (kFxWeak) go through near_centre_fp64 whole, with the arithmetic's own infinities
+// and NaN.
 #include <math.h>
 
 #include <type_traits>
@@ -43,6 +43,22 @@ constexpr int kFxWarps = kNearThreads / 32;
 // a source's strength: S (h, l) [62]; D (re.h, re.l, im.h, im.l) [60], split at bit 30
 template <int KERNEL> struct FxStr { typedef int2 T; };
 template <> struct FxStr<GQ_D> { typedef int4 T; };
+
+// Where a centre's terms are weak beside the largest strength of the tile (panels of
+// very different length in one box), the common scale leaves them fewer bits than
+// FP64's: at n sources the sum's rounding, about sqrt(n) 2^-60 of that strength, has to
+// stay below 2^-53 of the sum of the terms' magnitudes, or the centre goes through
+// near_centre_fp64.  The bound on that sum in units of 2^-22 of the scale is
+// kFxWeak sqrt(n).  Errors against long double, q = 5 .. 16, one panel and another 2^k
+// times longer (host build of gq_fix.cuh): S equal at 2^11, 10 times FP64's at 2^14;
+// D at 2^8 and 2^11; this bound cuts at 2^9 and 2^7.  Panels of one length are 14 to 80
+// times above it.  Cost, 64 circles with panels graded over 2^20, q = 8, D: n_max 32 2.51 ->
+// 2.74 ms (all in FP64: 9.6), n_max 256 and 16 nodes a panel, where nearly all centres
+// mix 2^9 and more, 5.0 -> 18.3 (17.1).
+constexpr float kFxWeak = 107021.0f;   // 2^21 at 384 sources
+
+__device__ __forceinline__ int fx_second(int2) { return 0; }
+__device__ __forceinline__ int fx_second(int4 v) { return v.z; }
 
 // -1/m
 __constant__ double c_ninv[GQ_MAX_PQBX + 1] = {0.0,      -1.0,      -1.0 / 2,  -1.0 / 3,  -1.0 / 4,  -1.0 / 5,
@@ -140,10 +156,11 @@ __device__ __noinline__ void near_centre_fp64(const EvalView &E, const NearRange
 // Stage the sources [v0, v1) of the loaded ranges: positions, and strengths as
 // q 2^(1022 - qe) <= 1/2 (D: each component, so that |d| <= 0.36) with qe from the
 // tile's largest exponent; for S the sums of the strengths' words per warp.
-// Returns qe, 0 where the strengths have no scale; ends with a barrier.
+// Returns qe, 0 where the strengths have no scale; ends with a barrier.  any: not all
+// strengths are zero.
 template <int KERNEL>
 __device__ __forceinline__ int fx_stage(const EvalView &E, const NearRanges &R, int v0, int v1, double2 *sy,
-                                        typename FxStr<KERNEL>::T *sq, long long *ssum, int *smax) {
+                                        typename FxStr<KERNEL>::T *sq, long long *ssum, int *smax, bool &any) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int mx = 0;
     for (int r = w; r < R.n; r += kFxWarps) {   // a warp takes one range at a time
@@ -159,7 +176,8 @@ __device__ __forceinline__ int fx_stage(const EvalView &E, const NearRanges &R, 
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kFxWarps; ++k) mx = max(mx, smax[k]);
-    if (mx == 0) mx = 1023;   // all zero
+    any = mx > 0;
+    if (!any) mx = 1023;
     const int qe = mx + (KERNEL == GQ_D ? 2 : 1);
     long long sh = 0, sl = 0;
     for (int r = w; r < R.n; r += kFxWarps) {
@@ -242,8 +260,10 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
         for (int v0 = 0; v0 < T || first; v0 += kFxTile) {
             const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
             if (v0) __syncthreads();
-            const int qe = fx_stage<KERNEL>(E, R, v0, v1, sy, sq, ssum, smax);
+            bool any;
+            const int qe = fx_stage<KERNEL>(E, R, v0, v1, sy, sq, ssum, smax, any);
             const bool scaled = qe > 0;
+            const float amin = any ? kFxWeak * sqrtf((float)n) : 0.0f;
             for (int c = cb + w; c < ce; c += kFxWarps) {
                 const double2 cz = E.sc_xy[c];
                 const double rc = E.sc_r[c];
@@ -254,12 +274,13 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                 unsigned nlim = 0;   // terms of sources with an upper word of |w|^2 below it are formed in FP64
                 long long acc[NV];   // S: 0 the log sum, 1 unused, then Re, Im of each order; D: Re, Im of each order
                 unsigned nmin = 0xffffffffu, nmax = 0;   // upper words of |w|^2
+                unsigned am = 0;     // the lane's sum of |Re t| + |Im t|, t the term of order 1 (D: 0), upper words
                 auto sweep = [&](auto without) {
                     const uint64_t rb = fx_bits(re);
                     const gfx Rm = fx_bal((long long)(fx_mant(rb) << 9));
                     const int er = fx_expo(rb);
                     nmin = 0xffffffffu;
-                    nmax = 0;
+                    nmax = am = 0;
 #pragma unroll
                     for (int i = 0; i < NV; ++i) acc[i] = 0;
                     for (int v = lane; v < n; v += 32) {
@@ -271,7 +292,10 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                         if constexpr (KERNEL != GQ_D)
                             acc[0] += fx_mul(gfx{sv.x, sv.y}, fx_bal(fx_log_half(nb, eref, shl_, stj)));
                         const bool in = without.value && (unsigned)(nb >> 32) < nlim;
-                        if (in) sv = str_t{};
+                        if (in) {
+                            am += KERNEL == GQ_D ? (abs(sv.x) + abs(fx_second(sv))) >> 2 : abs(sv.x) >> 2;
+                            sv = str_t{};
+                        }
                         if (!in || KERNEL != GQ_D) nmin = min(nmin, (unsigned)(nb >> 32));
                         nmax = max(nmax, (unsigned)(nb >> 32));
                         gfx ux, uy, nuy;
@@ -288,6 +312,7 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                             acc[2] += tr;
                             acc[3] += ti;
                         }
+                        am += abs((int)(tr >> 32)) + abs((int)(ti >> 32));
 #pragma unroll
                         for (int m = KERNEL == GQ_D ? 1 : 2; m <= QQ; ++m) {
                             if (m % 4 == 0 && m > qc) break;
@@ -320,6 +345,18 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                     const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20), er = fx_expo(fx_bits(re));
                     slow = n > 0 && (emin < 128 || emax > 1920 || er < 128 || er > 1920 ||
                                      (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40)));
+                    // the centre's terms weak beside the tile's scale (kFxWeak)
+                    const float a = (float)__reduce_add_sync(0xffffffffu, am >> 6);
+                    if (!slow && !(a >= amin)) slow = true;
+                    else if (!slow && re != rc) {
+                        // the rounding grows as (rc/re)^m: either the first order or the last has to stand above it
+                        unsigned aq = 0;
+#pragma unroll
+                        for (int m = 1; m <= QQ; ++m)
+                            if (m == qc) aq = abs((int)(acc[2 * m] >> 32)) + abs((int)(acc[2 * m + 1] >> 32));
+                        const float g = powf((float)(rc / re), (float)(qc - 1));
+                        slow = a < amin * g && !((float)__reduce_add_sync(0xffffffffu, aq >> 6) >= amin);
+                    }
                 }
                 if (slow) {
                     near_centre_fp64<KERNEL>(E, R, v0, v1, cz, rc, QQ, qc, kAllSources, dst, first);
@@ -420,7 +457,8 @@ __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, con
         for (int v0 = 0; v0 < T || first; v0 += kFxTile) {
             const int v1 = min(T, v0 + kFxTile), n = v1 - v0;
             if (v0) __syncthreads();
-            const int qe = fx_stage<GQ_S>(E, R, v0, v1, sy, sq, ssum, smax);
+            bool any;
+            const int qe = fx_stage<GQ_S>(E, R, v0, v1, sy, sq, ssum, smax, any);
             const double sc = pow2_clamped(qe + 1 - 55);
             const double q0 = qe > 0 ? fx_strength_sum(ssum) * (sc * 0x1p-7) * ((eref - 1023) * 0.34657359027997264) : 0.0;
             // the sums of up to 32 targets wait in the lanes and are converted together

@@ -67,3 +67,41 @@ def test_many_sources_inside_the_disk(kern, count):
     g["up_w"] = g["up_w"].copy()
     g["up_w"][src] *= np.resize([0.0, 1e-9, 1.0, 1e-3], count)
     assert _error(g, kern, 8, np.array([50, 51, 200])) <= 1
+
+
+def _graded(levels, nu, sides=2):
+    """A unit circle whose panels halve in length towards one point, from one side or
+    from both: neighbouring panels differ by 2 (at the point by up to 2^levels)."""
+    nb = 16
+    ref_b, ref_u, w_u = (np.polynomial.legendre.leggauss(n)[k] for n, k in ((nb, 0), (nu, 0), (nu, 1)))
+    up = np.pi * 0.5 ** np.arange(levels, -1, -1)
+    edges = np.concatenate([-up[::-1] if sides == 2 else np.linspace(-np.pi, 0, 9)[:-1], [0.0], up])
+    a, h = edges[:-1, None], np.diff(edges)[:, None] / 2
+
+    def nodes(ref):
+        th = (a + h + h * ref).ravel()
+        return np.stack([np.cos(th), np.sin(th)], 1)
+    w = (h * w_u).ravel()
+    b, u = nodes(ref_b), nodes(ref_u)
+    n = len(edges) - 1
+    density = np.random.default_rng(levels).normal(size=n * nb)
+    return dict(npanels=n, nb=nb, nu=nu, ref_b=ref_b, ref_u=ref_u, base_xy=b, base_n=b.copy(), up_xy=u, up_n=u.copy(),
+                up_w=w, panel_len=2 * h.ravel(), tgt_xy=b, tgt_onsurf=np.arange(n * nb, dtype=np.int32), density=density)
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+@pytest.mark.parametrize("levels,nu,sides", [(8, 16, 2), (16, 16, 2), (22, 16, 2), (22, 64, 2), (12, 24, 1), (20, 24, 1)])
+@pytest.mark.parametrize("q", [5, 16])
+def test_graded_panels_in_one_box(kern, levels, nu, sides, q):
+    g = _graded(levels, nu, sides)
+    assert _error(g, kern, q, np.arange(3, 2 * 16 * g["npanels"], 11)) <= 1
+
+
+def test_densities_with_zeros():
+    """Unit densities (one node of one panel) and none at all: tiles without strength."""
+    g = _problem(24)
+    for i in (0, 77):
+        g["density"] = np.zeros(24 * 16)
+        g["density"][i] = 1.0
+        for kern in ("S", "D"):
+            assert _error(g, kern, 8, np.arange(2 * (i // 16) * 16, 2 * (i // 16) * 16 + 32)) <= 1
