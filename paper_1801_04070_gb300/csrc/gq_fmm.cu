@@ -2099,6 +2099,12 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         SX.M = g->M2; SX.lvl = g->lvl2; SX.logt = T.dlogt; SX.H = (float)g->root.H;
         SX.near_pt = g->prm.eps < 1e-10;
     }
+    // Tiles and pairs of the tensor-core kernels that gq_build did not make (the orders
+    // were lowered since): here, on the context's stream, because their temporaries go
+    // back to the pool when they return, and what either side allocates after the fork
+    // may be one of those blocks.
+    if (g->n_far_boxes && !m2l_split && gq_m2l_tc_supported(g) && !g->tc_ready) gq_m2l_tc_build(g);
+    if (g->nc && !split_w && gq_w_tc_supported(g) && !g->wtc_ready) gq_w_tc_build(g);
     mark(S_STR, st);
     GQ_CUDA(cudaEventRecord(g->ev_str, st));
 
