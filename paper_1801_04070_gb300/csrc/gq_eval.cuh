@@ -137,16 +137,16 @@ void gq_near_centres_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *wo
 // direct potential at the point targets for S, likewise (gq_near_fx.cu)
 void gq_near_points_fx(gq_ctx *ctx, const EvalView &E, int nwork, const int *work, double *pot);
 // List 2 translations (M2L) of orders 16 .. 30 in fixed point (gq_m2l_fx.cu), added to L
-void gq_m2l_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *L);
+void gq_m2l_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double2 *L);
 void gq_m2l_fx_prepare(int dev);   // its tables on device dev
 // the multipoles of the boxes in fixed point, into g->Mfx and g->Efx (gq_w_fx.cu)
-void gq_mfix(gq_geom *g, int P1, const double2 *M);
+void gq_mfix(gq_geom *g, gq_ctx *ctx, int P1, const double2 *M);
 // List 3 far (gq_w_fx.cu), from g->Mfx and g->Efx: multipoles at the point targets, and to
 // the QBX centres for p_qbx <= kWFxMaxQ, added to pot and Q
 constexpr int kWFxMaxQ = 10;
-void gq_w_points_fx(gq_geom *g, const EvalView &E, const double2 *M, double *pot);
-void gq_w_centres_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *Q);
+void gq_w_points_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double *pot);
+void gq_w_centres_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double2 *Q);
 void gq_w_fx_prepare(int dev);     // its tables on device dev
 // M2M of all levels in fixed point (gq_m2m_fx.cu)
-void gq_m2m_fx(gq_geom *g, const EvalView &E, double2 *M);
+void gq_m2m_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, double2 *M);
 void gq_m2m_fx_prepare(int dev);   // its table on device dev

@@ -1953,8 +1953,12 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // batched evaluation does the direct parts and the final sums itself).
     const bool at_base = apply_identity != nullptr;
     const bool fmm_only = far != nullptr;
-    gq_ctx *ctx = g->ctx;
-    cudaStream_t st = ctx->stream;
+    // The evaluation's own copies of the context, one per stream: the context itself
+    // keeps its stream, for other threads' calls on it.
+    gq_ctx own = *g->ctx;
+    own.launches = 0;
+    gq_ctx *ctx = &own;
+    const cudaStream_t st = ctx->stream;
     EvalTables &T = get_tables(g);
     int P = g->prm.p_fmm, Qn = g->prm.p_qbx, P1 = P + 1, Q1 = Qn + 1;
     int kin = kernel == GQ_SP ? GQ_S : kernel;
@@ -2012,8 +2016,8 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // graph of many evaluations (12 geometries x 8 densities 35 -> 26 ms).  Either way
     // Stage 8 adds to its sums.
     const bool w_beside = !fmm_only && cap == cudaStreamCaptureStatusNone && g->nsrc < 800000;
-    gq_ctx ctx2 = *ctx;   // launches of the direct part
-    ctx2.launches = 0;
+    gq_ctx passes = *ctx;   // launches of the FMM passes
+    passes.stream = sf;
 
     // stage events (only when statistics are requested), kept with the geometry
     enum { S0, S_STR, S_FMM, S_M2M, S_M2L, S_P2L, S_L2L, S_S8, S_L2Q, S_WB, S_WC, S_WP, S_FIN, S_END, N_BEG, N_CTR, N_PT, NEV };
@@ -2026,7 +2030,6 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         if (timed) GQ_CUDA(cudaEventRecord(ev[i], on));
     };
     mark(S0, st);
-    int64_t l0 = ctx->launches;
 
     // A1
     GQ_CUDA(cudaMemsetAsync(g->qexp.p, 0, sizeof(unsigned int), st));
@@ -2111,28 +2114,28 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // ---- Stages 3, 5a, 6a (direct interactions)
     mark(N_BEG, st);
     if (g->n_ctr_boxes && !fmm_only) {
-        if (f32) dispatch_near_centres_f32(&ctx2, E, X, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
+        if (f32) dispatch_near_centres_f32(ctx, E, X, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
         // the FP32-pair tier too: fixed point is faster than pairs (1.05 M nodes, q = 4: 3.18 ms in pairs) and
         // closer to 64 bits
-        else gq_near_centres_fx(&ctx2, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
+        else gq_near_centres_fx(ctx, E, g->n_ctr_boxes, g->ctr_boxes, g->Qn.p);
     }
     mark(N_CTR, st);
     if (g->n_pt_boxes && !at_base && !fmm_only) {
         if (f32) {
             auto kd = k_near_points_f32<GQ_D>;
             auto ks = k_near_points_f32<GQ_S>;
-            GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, X, g->n_pt_boxes,
+            GQ_LAUNCH(ctx, (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, X, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
         } else if (split) {   // pairs: 0.72 ms where fixed point takes 0.78 (0.86 M targets)
             auto kd = k_near_points_split<GQ_D>;
             auto ks = k_near_points_split<GQ_S>;
-            GQ_LAUNCH((&ctx2), (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, SX, g->n_pt_boxes,
+            GQ_LAUNCH(ctx, (kin == GQ_D ? kd : ks), g->n_pt_boxes, kNearThreads, 0, E, SX, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
         } else if (kin == GQ_D) {
-            GQ_LAUNCH((&ctx2), k_near_points<GQ_D>, g->n_pt_boxes, kNearThreads, 0, E, g->n_pt_boxes,
+            GQ_LAUNCH(ctx, k_near_points<GQ_D>, g->n_pt_boxes, kNearThreads, 0, E, g->n_pt_boxes,
                       (const int *)g->pt_boxes, g->potn.p);
         } else {
-            gq_near_points_fx(&ctx2, E, g->n_pt_boxes, g->pt_boxes, g->potn.p);
+            gq_near_points_fx(ctx, E, g->n_pt_boxes, g->pt_boxes, g->potn.p);
         }
     }
     mark(N_PT, st);
@@ -2141,39 +2144,36 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     const bool m2l_fx = !m2l_split && P1 > 16;
     const bool wc_fx = !split_w && g->nc > 0 && !gq_w_tc_supported(g) && Qn <= kWFxMaxQ;
     const bool wp_fx = !f32 && !split_w && g->npt > 0 && !at_base;
-    // Stage 5b, on the stream that the context's launches go to
-    auto list3_far = [&]() {
-        mark(S_WB, ctx->stream);
+    // Stage 5b on the stream of c
+    auto list3_far = [&](gq_ctx *c) {
+        mark(S_WB, c->stream);
         if (g->nc && split_w) {
-            dispatch_w_centres_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
+            dispatch_w_centres_split(c, E, SX, g->nc, (const int *)g->ctr_owner, Qb);
         } else if (g->nc) {
-            if (gq_w_tc_supported(g)) gq_w_centres_tc(g, E.R, (const double2 *)g->M, T.logt, Qb);
-            else if (wc_fx) gq_w_centres_fx(g, E, (const double2 *)g->M, Qb);
-            else dispatch_w_centres_q(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
+            if (gq_w_tc_supported(g)) gq_w_centres_tc(g, c, E.R, (const double2 *)g->M, T.logt, Qb);
+            else if (wc_fx) gq_w_centres_fx(g, c, E, (const double2 *)g->M, Qb);
+            else dispatch_w_centres_q(c, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->M, Qb);
         }
-        mark(S_WC, ctx->stream);
+        mark(S_WC, c->stream);
         if (g->npt && !at_base) {
             if (f32)
-                GQ_LAUNCH(ctx, k_w_points_f32, gq_blocks(g->npt, 128), 128, 0, E, X, g->npt, (const int *)g->pt_owner,
+                GQ_LAUNCH(c, k_w_points_f32, gq_blocks(g->npt, 128), 128, 0, E, X, g->npt, (const int *)g->pt_owner,
                           potb);
             else if (split_w)
-                GQ_LAUNCH(ctx, k_w_points_split, gq_blocks(g->npt, 128), 128, 0, E, SX, g->npt, (const int *)g->pt_owner,
+                GQ_LAUNCH(c, k_w_points_split, gq_blocks(g->npt, 128), 128, 0, E, SX, g->npt, (const int *)g->pt_owner,
                           potb);
             else
-                gq_w_points_fx(g, E, (const double2 *)g->M, potb);
+                gq_w_points_fx(g, c, E, (const double2 *)g->M, potb);
         }
-        mark(S_WP, ctx->stream);
+        mark(S_WP, c->stream);
     };
 
-    // ---- FMM passes: the context's launches go to their stream until the join
-    // (an exception waits for them: the geometry's buffers are then unused)
-    struct OnStream {
-        gq_ctx *c;
-        cudaStream_t own, s;
+    // ---- FMM passes (an exception waits for them: the geometry's buffers are then unused)
+    struct Drain {
+        cudaStream_t s;
         int depth = std::uncaught_exceptions();
-        OnStream(gq_ctx *c_, cudaStream_t s_) : c(c_), own(c_->stream), s(s_) { c->stream = s_; }
-        ~OnStream() {
-            c->stream = own;
+        explicit Drain(cudaStream_t s_) : s(s_) {}
+        ~Drain() {
             if (std::uncaught_exceptions() > depth) {
                 cudaStreamSynchronize(s);
                 cudaGetLastError();
@@ -2181,7 +2181,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         }
     };
     {
-    OnStream passes(ctx, sf);
+    Drain drain(sf);
     GQ_CUDA(cudaStreamWaitEvent(sf, g->ev_str, 0));
     mark(S_FMM, sf);
     GQ_CUDA(cudaMemsetAsync(g->M.p, 0, sizeof(double2) * g->nbox * P1, sf));
@@ -2199,34 +2199,34 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             auto k8 = k_p2m_split<8>;
             auto k16 = k_p2m_split<16>;
             auto k32 = k_p2m_split<GQ_MAX_PFMM>;
-            GQ_LAUNCH(ctx, (P <= 8 ? k8 : P <= 16 ? k16 : k32), gq_blocks((long long)g->n_leaf_src * kP2MG, 128),
+            GQ_LAUNCH(&passes, (P <= 8 ? k8 : P <= 16 ? k16 : k32), gq_blocks((long long)g->n_leaf_src * kP2MG, 128),
                       128, 0, E, SX, g->n_leaf_src, (const int *)g->leaf_src_boxes, g->M2.p);
         } else {
             auto k8 = k_p2m<8>;
             auto k16 = k_p2m<16>;
             auto k32 = k_p2m<GQ_MAX_PFMM>;
-            GQ_LAUNCH(ctx, (P <= 8 ? k8 : P <= 16 ? k16 : k32), gq_blocks((long long)g->n_leaf_src * kP2MG, 128),
+            GQ_LAUNCH(&passes, (P <= 8 ? k8 : P <= 16 ? k16 : k32), gq_blocks((long long)g->n_leaf_src * kP2MG, 128),
                       128, 0, E, g->n_leaf_src, (const int *)g->leaf_src_boxes, g->M.p);
         }
     }
     if (m2l_split)
         for (int l = g->nlev - 2; l >= 0; --l) {
             const int s = g->level_start_h[l], e = g->level_start_h[l + 1];
-            GQ_LAUNCH(ctx, k_m2m_split, gq_blocks((long long)(e - s) * P1, 128), 128, 0, E, s, e, T.tm2m2, g->M2.p);
+            GQ_LAUNCH(&passes, k_m2m_split, gq_blocks((long long)(e - s) * P1, 128), 128, 0, E, s, e, T.tm2m2, g->M2.p);
         }
     else
-        gq_m2m_fx(g, E, g->M.p);
+        gq_m2m_fx(g, &passes, E, g->M.p);
     mark(S_M2M, sf);
     if (m2l_split)
-        GQ_LAUNCH(ctx, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+        GQ_LAUNCH(&passes, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const float4 *)g->M2, g->M.p);
     else if (split_w)   // multipoles as FP32 pairs for the pair List 3 far kernels
-        GQ_LAUNCH(ctx, k_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+        GQ_LAUNCH(&passes, k_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->M, g->M2.p);
     // the multipoles in fixed point for the kernels that work there
-    if (m2l_fx || wc_fx || wp_fx) gq_mfix(g, P1, (const double2 *)g->M);
+    if (m2l_fx || wc_fx || wp_fx) gq_mfix(g, &passes, P1, (const double2 *)g->M);
     if (f32)
-        GQ_LAUNCH(ctx, k_to_float2, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+        GQ_LAUNCH(&passes, k_to_float2, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->M, g->M_f.p);
     GQ_CUDA(cudaEventRecord(g->ev_m2m, sf));
     // Stage 4
@@ -2236,15 +2236,15 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
             size_t sm = sizeof(float2) * P1 * (P1 | 1);
             auto k16 = k_m2l_split<16>;
             auto k32 = k_m2l_split<32>;
-            GQ_LAUNCH(ctx, (G == 16 ? k16 : k32), gq_blocks((long long)g->n_far_boxes * G, 128), 128, sm, E, SX,
+            GQ_LAUNCH(&passes, (G == 16 ? k16 : k32), gq_blocks((long long)g->n_far_boxes * G, 128), 128, sm, E, SX,
                       g->n_far_boxes, (const int *)g->far_boxes, T.dtab2, T.logtab2, T.binom2, g->L2.p);
         } else if (gq_m2l_tc_supported(g)) {
-            gq_m2l_tc(g, (const double2 *)g->M, g->L.p);   // FP64-accurate, on the tensor cores
+            gq_m2l_tc(g, &passes, (const double2 *)g->M, g->L.p);   // FP64-accurate, on the tensor cores
         } else if (m2l_fx) {
-            gq_m2l_fx(g, E, (const double2 *)g->M, g->L.p);   // in fixed point
+            gq_m2l_fx(g, &passes, E, (const double2 *)g->M, g->L.p);   // in fixed point
         } else {
             auto k16 = k_m2l<16>;
-            GQ_LAUNCH(ctx, k16, gq_blocks((long long)g->n_far_boxes * 16, 128), 128, sizeof(double) * P1 * P1, E,
+            GQ_LAUNCH(&passes, k16, gq_blocks((long long)g->n_far_boxes * 16, 128), 128, sizeof(double) * P1 * P1, E,
                       g->n_far_boxes, (const int *)g->far_boxes, (const double2 *)g->M, (const double2 *)T.dtab,
                       (const double *)T.logtab, g->L.p);
         }
@@ -2252,46 +2252,44 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     mark(S_M2L, sf);
     if (g->n_far_boxes) {
         // Stage 6b
-        GQ_LAUNCH(ctx, k_p2l, gq_blocks((long long)g->n_far_boxes * 32, 128), 128, 0, E, g->n_far_boxes,
+        GQ_LAUNCH(&passes, k_p2l, gq_blocks((long long)g->n_far_boxes * 32, 128), 128, 0, E, g->n_far_boxes,
                   (const int *)g->far_boxes, g->L.p);
     }
     mark(S_P2L, sf);
     // Stage 7 (in pairs wherever M2L runs in pairs: the FP64 P2L terms are
     // folded into the pair locals first, and the FP64 copy is made at the end)
     if (m2l_split)
-        GQ_LAUNCH(ctx, k_add_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+        GQ_LAUNCH(&passes, k_add_to_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const double2 *)g->L, g->L2.p);
     for (int l = 1; l < g->nlev; ++l) {
         int s = g->level_start_h[l], e = g->level_start_h[l + 1];
         if (m2l_split)
-            GQ_LAUNCH(ctx, k_l2l_split, gq_blocks((long long)(e - s) * P1, 128), 128, 0, E, s, e, T.tl2l2, g->L2.p);
+            GQ_LAUNCH(&passes, k_l2l_split, gq_blocks((long long)(e - s) * P1, 128), 128, 0, E, s, e, T.tl2l2, g->L2.p);
         else
-            GQ_LAUNCH(ctx, k_l2l_t, gq_blocks(e - s, 128 / P1), (128 / P1) * P1, 0, E, s, e,
+            GQ_LAUNCH(&passes, k_l2l_t, gq_blocks(e - s, 128 / P1), (128 / P1) * P1, 0, E, s, e,
                       (const double2 *)T.tl2l, g->L.p);
     }
     if (m2l_split)
-        GQ_LAUNCH(ctx, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
+        GQ_LAUNCH(&passes, k_from_dfl4, gq_blocks((long long)g->nbox * P1, 256), 256, 0, (long long)g->nbox * P1,
                   (const float4 *)g->L2, g->L.p);
     mark(S_L2L, sf);
     if (w_beside) {
-        ctx->stream = st;
         GQ_CUDA(cudaStreamWaitEvent(st, g->ev_m2m, 0));
-        list3_far();
+        list3_far(ctx);
         GQ_CUDA(cudaEventRecord(g->ev_w, st));
-        ctx->stream = sf;
         GQ_CUDA(cudaStreamWaitEvent(sf, g->ev_w, 0));
     } else {
-        list3_far();
+        list3_far(&passes);
     }
     mark(S_S8, sf);
     // Stage 8
     if (g->nc)
         if (m2l_split)
-            dispatch_l2qbxl_split(ctx, E, SX, g->nc, (const int *)g->ctr_owner, (const float4 *)g->L2, Qb);
+            dispatch_l2qbxl_split(&passes, E, SX, g->nc, (const int *)g->ctr_owner, (const float4 *)g->L2, Qb);
         else
-            dispatch_l2qbxl_t(ctx, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->L, Qb);
+            dispatch_l2qbxl_t(&passes, E, g->nc, (const int *)g->ctr_owner, (const double2 *)g->L, Qb);
     if (g->npt && !at_base)
-        GQ_LAUNCH(ctx, k_l2p, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner, (const double2 *)g->L,
+        GQ_LAUNCH(&passes, k_l2p, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner, (const double2 *)g->L,
                   potb);
     mark(S_L2Q, sf);
     GQ_CUDA(cudaEventRecord(g->ev_fmm, sf));
@@ -2314,7 +2312,8 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
                   (const double *)g->sc_r, (const double2 *)g->Q, (const double2 *)g->Qn, (const double *)g->pot,
                   (const double *)g->potn, out_dev);
     mark(S_END, st);
-    ctx->launches += ctx2.launches;
+    const int64_t launches = ctx->launches + passes.launches;
+    g->ctx->launches += launches;
     if (timed) {
         GQ_CUDA(cudaEventSynchronize(ev[S_END]));
         {
@@ -2339,7 +2338,7 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
         stt->ms_stage[8] = el(S_WC, S_WP);
         stt->ms_stage[9] = el(S_S8, S_L2Q);
         stt->ms_stage[10] = el(S_FIN, S_END);
-        stt->kernel_launches = ctx->launches - l0;
+        stt->kernel_launches = launches;
     }
     g->have_eval = true;
     g->last_kernel = kernel;

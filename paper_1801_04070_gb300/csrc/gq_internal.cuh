@@ -254,13 +254,13 @@ void gq_bplan_fmm(gq_bplan *P, int i);
 void gq_bplan_persistent(gq_bplan *P, gq_ctx *ctx, int grid, unsigned long long limit_ns);
 int gq_bplan_error(gq_bplan *P);
 bool gq_m2l_tc_supported(const gq_geom *g);                                                  // gq_m2l_tc.cu
-void gq_m2l_tc(gq_geom *g, const double2 *M, double2 *L);
+void gq_m2l_tc(gq_geom *g, gq_ctx *ctx, const double2 *M, double2 *L);
 void gq_m2l_tc_build(gq_geom *g);
 int gq_m2l_tc_error(gq_geom *g);
 bool gq_w_tc_supported(const gq_geom *g);
 void gq_tensor_paths_impl(gq_geom *g, int *m2l_tc, int *m2qbxl_tc);
 void gq_w_tc_build(gq_geom *g);
-void gq_w_centres_tc(gq_geom *g, const RootInfo &R, const double2 *M, const double *logt, double2 *Q);
+void gq_w_centres_tc(gq_geom *g, gq_ctx *ctx, const RootInfo &R, const double2 *M, const double *logt, double2 *Q);
 struct gq_mlp;
 int gq_mlp_param_count();                                                                   // gq_learned.cu
 gq_mlp *gq_mlp_new(gq_ctx *ctx, uint64_t seed);

@@ -179,10 +179,10 @@ const M2LFxTables &tables(int dev) {
 
 }  // namespace
 
-void gq_m2l_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *L) {
-    const M2LFxTables &T = tables(g->ctx->device);
+void gq_m2l_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double2 *L) {
+    const M2LFxTables &T = tables(ctx->device);
     const int blocks = gq_blocks(g->n_far_boxes, kM2LWarps);
-    GQ_LAUNCH(g->ctx, k_m2l_fx, blocks < 152 * 32 ? blocks : 152 * 32, kM2LWarps * 32, 0, E, g->n_far_boxes,
+    GQ_LAUNCH(ctx, k_m2l_fx, blocks < 152 * 32 ? blocks : 152 * 32, kM2LWarps * 32, 0, E, g->n_far_boxes,
               (const int *)g->far_boxes, M, (const longlong2 *)g->Mfx, (const int *)g->Efx, T.c, T.d, T.s, T.logd, L);
 }
 

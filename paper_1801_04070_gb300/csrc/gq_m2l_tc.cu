@@ -608,8 +608,7 @@ void gq_m2l_tc_build(gq_geom *g) {
 }
 
 // M2L of the current multipoles M into L (added) on the tensor cores.
-void gq_m2l_tc(gq_geom *g, const double2 *M, double2 *L) {
-    gq_ctx *ctx = g->ctx;
+void gq_m2l_tc(gq_geom *g, gq_ctx *ctx, const double2 *M, double2 *L) {
     GQ_REQUIRE(g->tc_ready, GQ_ERR_STATE, "tensor-core M2L before its tiles");
     const TcConst &T = tc_const(ctx->device);
     const int nbox = g->nbox, P = g->prm.p_fmm;

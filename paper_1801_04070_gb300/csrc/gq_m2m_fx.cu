@@ -144,12 +144,12 @@ const int4 *table(int dev) {
 
 void gq_m2m_fx_prepare(int dev) { table(dev); }
 
-void gq_m2m_fx(gq_geom *g, const EvalView &E, double2 *M) {
-    const int4 *T = table(g->ctx->device);
+void gq_m2m_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, double2 *M) {
+    const int4 *T = table(ctx->device);
     const int bpb = kM2MThreads / (E.P + 1);
     for (int l = g->nlev - 2; l >= 0; --l) {
         const int s = g->m2m_level_start_h[l], e = g->m2m_level_start_h[l + 1];
         if (e > s)
-            GQ_LAUNCH(g->ctx, k_m2m_fx, gq_blocks(e - s, bpb), kM2MThreads, 0, E, (const int *)g->m2m_boxes, s, e, T, M);
+            GQ_LAUNCH(ctx, k_m2m_fx, gq_blocks(e - s, bpb), kM2MThreads, 0, E, (const int *)g->m2m_boxes, s, e, T, M);
     }
 }

@@ -253,23 +253,23 @@ const WFxTables &tables(int dev) {
 
 void gq_w_fx_prepare(int dev) { tables(dev); }
 
-void gq_mfix(gq_geom *g, int P1, const double2 *M) {
+void gq_mfix(gq_geom *g, gq_ctx *ctx, int P1, const double2 *M) {
     g->Mfx.alloc((size_t)g->nbox * P1);
     g->Efx.alloc(g->nbox);
-    GQ_LAUNCH(g->ctx, k_mfix, gq_blocks((long long)g->nbox * 32, 256), 256, 0, g->nbox, P1, M, g->Mfx.p, g->Efx.p);
+    GQ_LAUNCH(ctx, k_mfix, gq_blocks((long long)g->nbox * 32, 256), 256, 0, g->nbox, P1, M, g->Mfx.p, g->Efx.p);
 }
 
-void gq_w_points_fx(gq_geom *g, const EvalView &E, const double2 *M, double *pot) {
-    GQ_LAUNCH(g->ctx, k_w_points_fx, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner, M,
+void gq_w_points_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double *pot) {
+    GQ_LAUNCH(ctx, k_w_points_fx, gq_blocks(g->npt, 128), 128, 0, E, g->npt, (const int *)g->pt_owner, M,
               (const longlong2 *)g->Mfx, (const int *)g->Efx, pot);
 }
 
-void gq_w_centres_fx(gq_geom *g, const EvalView &E, const double2 *M, double2 *Q) {
-    const WFxTables W = tables(g->ctx->device);
+void gq_w_centres_fx(gq_geom *g, gq_ctx *ctx, const EvalView &E, const double2 *M, double2 *Q) {
+    const WFxTables W = tables(ctx->device);
     switch (E.Q) {
 #define GQ_CASE(v)                                                                                                     \
     case v:                                                                                                            \
-        GQ_LAUNCH(g->ctx, k_w_centres_fx<v>, gq_blocks(g->nc, 128), 128, 0, E, g->nc, (const int *)g->ctr_owner, M,    \
+        GQ_LAUNCH(ctx, k_w_centres_fx<v>, gq_blocks(g->nc, 128), 128, 0, E, g->nc, (const int *)g->ctr_owner, M,    \
                   (const longlong2 *)g->Mfx, (const int *)g->Efx, W, Q);                                               \
         break;
         GQ_CASE(1) GQ_CASE(2) GQ_CASE(3) GQ_CASE(4) GQ_CASE(5) GQ_CASE(6) GQ_CASE(7) GQ_CASE(8) GQ_CASE(9) GQ_CASE(10)

@@ -508,8 +508,7 @@ void gq_w_tc_build(gq_geom *g) {
 }
 
 // M2QBXL of the multipoles M into the (sorted-centre) QBX coefficients Q (added).
-void gq_w_centres_tc(gq_geom *g, const RootInfo &R, const double2 *M, const double *logt, double2 *Q) {
-    gq_ctx *ctx = g->ctx;
+void gq_w_centres_tc(gq_geom *g, gq_ctx *ctx, const RootInfo &R, const double2 *M, const double *logt, double2 *Q) {
     GQ_REQUIRE(g->wtc_ready, GQ_ERR_STATE, "tensor-core M2QBXL before its pairs");
     const int P = g->prm.p_fmm, q = g->prm.p_qbx;
     const WConst &T = w_const(ctx->device, P, q);
