@@ -126,10 +126,15 @@ __device__ __forceinline__ void warp_reduce_scatter(V (&v)[NV], V zero, int lane
 // ------------------------------------------------------------------ multipoles in fixed point
 // exponent of a box whose multipoles are not all finite
 constexpr int kFxNaNExp = 1 << 20;
-static __device__ __forceinline__ double fx_scale_of(int E) {   // 2^(E - 1022)
-    if (E == kFxNaNExp) return __longlong_as_double(0x7ff8000000000000ll);
-    return E + 1 >= 1 ? (E + 1 <= 2046 ? __longlong_as_double((long long)(E + 1) << 52) : 2.0 * __longlong_as_double(2046ll << 52))
-                      : ldexp(1.0, max(E - 1022, -1100));
+// The scale 2^(x - 1023) of v.  Where it is no normal number v is scaled instead, in two
+// steps that round once, and the scale is 1 (strengths near the ends of the range,
+// whose sums are still finite); NaN for a box of kFxNaNExp.
+static __device__ __forceinline__ double fx_scale(double &v, int x) {
+    if ((unsigned)(x - 1) < 2046u) return __longlong_as_double((long long)x << 52);
+    const int n = max(x - 1023, -1500), h = n >> 1;   // (a box of zeros: far below)
+    if (x > kFxNaNExp / 2) v = __longlong_as_double(0x7ff8000000000000ll);
+    else v = v * __longlong_as_double((long long)(h + 1023) << 52) * __longlong_as_double((long long)(n - h + 1023) << 52);
+    return 1.0;
 }
 
 // direct sums to the QBX centres in 64-bit fixed point (gq_near_fx.cu): Qout [nc][E.Q+1]

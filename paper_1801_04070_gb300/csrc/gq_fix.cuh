@@ -104,11 +104,19 @@ GQ_HD uint64_t fx_shr(uint64_t v, int s) {
 GQ_HD uint64_t fx_mant(uint64_t bits) { return (bits & 0xfffffffffffffull) | 0x10000000000000ull; }
 GQ_HD int fx_expo(uint64_t bits) { return (int)(bits >> 52) & 0x7ff; }
 
+// the biased exponent of x: 0 for zero only (1 for a subnormal number)
+GQ_HD int fx_expo1(double x) {
+    const uint64_t b = fx_bits(x);
+    const int e = fx_expo(b);
+    return e > 0 ? e : (b << 1) != 0;
+}
+
 // x 2^(1022 - e) 2^62 for |x| < 2^(e - 1022) (e: a biased exponent no smaller than x's), truncated
 GQ_HD long long fx_from_double(double x, int e) {
     const uint64_t b = fx_bits(x);
     const int ex = fx_expo(b);
-    const long long v = ex ? (long long)fx_shr(fx_mant(b) << 10, e + 1 - ex) : 0;
+    const uint64_t m = ex ? fx_mant(b) : b & 0xfffffffffffffull;
+    const long long v = (long long)fx_shr(m << 10, e + 1 - (ex ? ex : 1));
     return (long long)b < 0 ? -v : v;
 }
 

@@ -85,8 +85,11 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_m2l_fx(EvalView E, int nwork
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 if (j + p >= end) break;
-                const double s = fx_scale_of(Ef[dd[p]]);
-                const double2 t = make_double2((double)(hr[p] + (int)(mr[p] >> 32)) * s, (double)(hi[p] + (int)(mi[p] >> 32)) * s);
+                double2 t = make_double2((double)(hr[p] + (int)(mr[p] >> 32)), (double)(hi[p] + (int)(mi[p] >> 32)));
+                const int e = Ef[dd[p]] + 1 - 56;
+                const double sx = fx_scale(t.x, e), sy = fx_scale(t.y, e);
+                t.x *= sx;
+                t.y *= sy;
                 const double2 f = stab[off[p] * 32 + m];
                 // the entry's own terms first: one rounding of the running sum an entry
                 const double lg = m == 0 ? M[(size_t)dd[p] * P1].x * (logrho + logtab[off[p]]) : 0.0;
@@ -104,7 +107,7 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_m2l_fx(EvalView E, int nwork
 struct M2LFxTables {
     const int2 *c = nullptr;        // [kP1][32] c_mk [62]: entry k * 32 + m
     const int4 *d = nullptr;        // [121][32] (4/delta)^k [62]
-    const double2 *s = nullptr;     // [121][32] (-1)^m delta^-m 2^(e_m - 56)
+    const double2 *s = nullptr;     // [121][32] (-1)^m delta^-m 2^e_m
     const double *logd = nullptr;   // [121] log|delta|
 };
 
@@ -158,7 +161,7 @@ const M2LFxTables &tables(int dev) {
             for (int k = 0; k < kP1; ++k) {
                 const int2 x = words(pr), y = words(pi);
                 d[off * 32 + k] = make_int4(x.x, x.y, y.x, y.y);
-                const long double f = ldexpl(k & 1 ? -1.0L : 1.0L, em[k] - 56 - 2 * k);
+                const long double f = ldexpl(k & 1 ? -1.0L : 1.0L, em[k] - 2 * k);
                 s[off * 32 + k] = make_double2((double)(f * pr), (double)(f * pi));
                 const long double nr = 4.0L * (pr * re + pi * im) / n2;
                 pi = 4.0L * (pi * re - pr * im) / n2;

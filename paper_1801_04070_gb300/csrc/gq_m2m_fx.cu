@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kM2MThreads) k_m2m_fx(EvalView E, const int *_
         if (i0 + bb >= lend) continue;
         const int c = child_of(E.bchild[boxes[i0 + bb]], q);
         if (c >= 0) v[r] = M[(size_t)c * P1 + k];
-        const int e = max(fx_expo(fx_bits(v[r].x)), fx_expo(fx_bits(v[r].y)));
+        const int e = max(fx_expo1(v[r].x), fx_expo1(v[r].y));
         if (e) atomicMax(&sE[bb], e - (k + 1) / 2 + (e == 0x7ff ? 4096 : 0));   // infinite or NaN: above any scale
     }
     __syncthreads();
@@ -88,8 +88,10 @@ __global__ void __launch_bounds__(kM2MThreads) k_m2m_fx(EvalView E, const int *_
     } else if (Eb < -2000) {   // no multipole at all
         out.x = out.y = 0.0;
     } else {
-        const double s = fx_scale_of(Eb + (m + 1) / 2) * 0x1p-60;
-        out = make_double2((double)sr * s, m ? (double)si * s : 0.0);
+        double x = (double)sr, y = (double)si;
+        const int e = Eb + (m + 1) / 2 + 1 - 60;
+        const double sx = fx_scale(x, e), sy = fx_scale(y, e);
+        out = make_double2(x * sx, m ? y * sy : 0.0);
     }
     M[(size_t)b * P1 + m] = out;
 }

@@ -72,12 +72,6 @@ __device__ __forceinline__ double pow2_clamped(int e) {
                              : e > -52 ? __longlong_as_double(1ll << (51 + e)) : 0.0;
 }
 
-// biased exponent of a strength: 0 for zero only (1 for a subnormal)
-__device__ __forceinline__ int str_expo(double x) {
-    const int e = fx_expo(fx_bits(x));
-    return e > 0 ? e : x != 0.0;
-}
-
 // The lane and slot that hold entry i after a warp_reduce_scatter over n values.
 struct RsPlace {
     int lane, slot;
@@ -167,8 +161,8 @@ __device__ __forceinline__ int fx_stage(const EvalView &E, const NearRanges &R, 
         const int p0 = R.pre[r], p1 = R.pre[r + 1];
         for (int v = max(p0, v0) + lane; v < min(p1, v1); v += 32) {
             const double2 st = E.str[R.beg[r] + (v - p0)];
-            mx = max(mx, str_expo(st.x));
-            if (KERNEL == GQ_D) mx = max(mx, str_expo(st.y));
+            mx = max(mx, fx_expo1(st.x));
+            if (KERNEL == GQ_D) mx = max(mx, fx_expo1(st.y));
         }
     }
     mx = __reduce_max_sync(0xffffffffu, mx);

@@ -36,7 +36,7 @@ __global__ void k_mfix(int nbox, int P1, const double2 *__restrict__ M, longlong
     if (b >= nbox) return;
     const bool act = k < P1;
     const double2 A = act ? M[(size_t)b * P1 + k] : make_double2(0.0, 0.0);
-    const int e = max(fx_expo(fx_bits(A.x)), fx_expo(fx_bits(A.y)));
+    const int e = max(fx_expo1(A.x), fx_expo1(A.y));
     const int kc = (k + 1) / 2;
     const int E = __reduce_max_sync(0xffffffffu, e ? e - kc : -1000);
     const bool bad = __any_sync(0xffffffffu, e == 0x7ff);
@@ -98,8 +98,9 @@ __global__ void __launch_bounds__(128) k_w_points_fx(EvalView E, int npt, const 
             hi = im + A1.y;
         }
         fx_cmul30(fx_split30(hr), fx_split30(hi), x2, y2, ny2, re, im);
-        const double s = fx_scale_of(Ef[d]) * 0x1p-58;
-        acc += fma((double)re, s, M[(size_t)d * P1].x * fx_log_abs(nb, fx_expo(rb), hl, tj));
+        double h = (double)re;
+        const double s = fx_scale(h, Ef[d] + 1 - 58);
+        acc += fma(h, s, M[(size_t)d * P1].x * fx_log_abs(nb, fx_expo(rb), hl, tj));
     }
     pot[t] += acc;
 }
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(128) k_w_centres_fx(EvalView E, int nc, const 
             }
         }
         // G_m / (S 2^em) [62] = the upper sum [56] and the middle one 32 bits below it
-        const double s = fx_scale_of(Ef[d]);
+        const int es = Ef[d] + 1;
         const int *em = W.em + (e - 1) * (kWFxMaxQ + 1);
         gfx ux, uy, nuy;   // -r/y
         fx_ratio(-yx, -yy, nb, fx_bal((long long)(fx_mant(rcb) << 9)), fx_expo(rcb), ux, uy, nuy);
@@ -188,10 +189,12 @@ __global__ void __launch_bounds__(128) k_w_centres_fx(EvalView E, int nc, const 
 #pragma unroll
         for (int m = 0; m <= QQ; ++m) {
             const long long gr = fx_shl(hr[m], 6) + (mr[m] >> 26), gi = fx_shl(hi[m], 6) + (mi[m] >> 26);
-            const double sm = s * __longlong_as_double((long long)(em[m] + 1023 - (m ? 60 : 62)) << 52);
+            const int e = es + em[m] - (m ? 60 : 62);   // the scale's exponent
             if (m == 0) {
-                acc[0].x += fma((double)gr, sm, M[(size_t)d * P1].x * fx_log_abs(nb, erho, hl, tj));
-                acc[0].y = fma((double)gi, sm, acc[0].y);
+                double x = (double)gr, y = (double)gi;
+                const double sx = fx_scale(x, e), sy = fx_scale(y, e);
+                acc[0].x += fma(x, sx, M[(size_t)d * P1].x * fx_log_abs(nb, erho, hl, tj));
+                acc[0].y = fma(y, sy, acc[0].y);
             } else {
                 long long re, im;
                 fx_cmul30(fx_split30(pr), fx_split30(pi), ux, uy, nuy, re, im);   // (-r/y)^m
@@ -199,8 +202,10 @@ __global__ void __launch_bounds__(128) k_w_centres_fx(EvalView E, int nc, const 
                 pi = im;
                 const gfx gx = fx_bal(gr | 1), gy = fx_bal(gi | 1);
                 fx_cmul30(fx_split30(pr), fx_split30(pi), gx, gy, gfx{-gy.h, -gy.l}, re, im);
-                acc[m].x = fma((double)re, sm, acc[m].x);
-                acc[m].y = fma((double)im, sm, acc[m].y);
+                double x = (double)re, y = (double)im;
+                const double sx = fx_scale(x, e), sy = fx_scale(y, e);
+                acc[m].x = fma(x, sx, acc[m].x);
+                acc[m].y = fma(y, sy, acc[m].y);
             }
         }
     }
