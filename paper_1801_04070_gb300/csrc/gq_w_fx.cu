@@ -46,9 +46,12 @@ __global__ void k_mfix(int nbox, int P1, const double2 *__restrict__ M, longlong
     if (k == 0) Ef[b] = bad ? kFxNaNExp : E;
 }
 
-// log|z| of |z|^2 = n2 (its bits), relative to rho = 2^(erho - 1023), plus log rho
+// log|z| of |z|^2 = n2 (its bits): relative to 1 while that fits the fixed point (64),
+// else to rho = 2^(erho - 1023) and plus log rho, which rounds at 2^-53 log rho also
+// where |z| is near 1.
 __device__ __forceinline__ double fx_log_abs(uint64_t nb, int erho, const long long *hl, const int *tj) {
-    return fma((double)fx_log_half(nb, 2 * erho - 1023, hl, tj), 0x1p-57, (erho - 1023) * 0.69314718055994531);
+    const int er = abs(fx_expo(nb) - 1023) <= 160 ? 1023 : 2 * erho - 1023;
+    return fma((double)fx_log_half(nb, er, hl, tj), 0x1p-57, (er - 1023) * 0.34657359027997264);
 }
 
 __global__ void __launch_bounds__(128) k_w_points_fx(EvalView E, int npt, const int *__restrict__ pt_owner,

@@ -105,3 +105,47 @@ def test_densities_with_zeros():
         g["density"][i] = 1.0
         for kern in ("S", "D"):
             assert _error(g, kern, 8, np.arange(2 * (i // 16) * 16, 2 * (i // 16) * 16 + 32)) <= 1
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+@pytest.mark.parametrize("levels", [12, 26])
+def test_small_far_boxes(kern, levels):
+    """List 3 far with boxes much smaller than their distance: strength only on the
+    smallest panels of a graded circle, seen from the large panels' centres (order 30,
+    k_w_centres_fx) and from points about 1 away, where log|z| is small (k_w_points_fx).
+    Tolerances: the sums of the 30 orders and of the levels round at 2^-53 of the
+    absolute sum each (70 in all); for S the potential is A_0 log|z| with |z| rounded at
+    2^-53 (and 1.75 with |z|^2 and the logarithm's own rounding)."""
+    from paper_1801_04070_gb300 import Geometry, params_default
+    from test_gpu_near_fixed import _strengths
+    g = _graded(levels, 32)
+    rng = np.random.default_rng(levels)
+    small = np.repeat(g["panel_len"] < 8 * g["panel_len"].min(), 16)
+    g["density"] = np.where(small, 2 + rng.normal(size=len(small)), 0.0)
+    a = rng.uniform(0, 2 * np.pi, 400)
+    g["tgt_xy"] = np.array([1.0, 0.0]) + rng.uniform(0.95, 1.05, (400, 1)) * np.stack([np.cos(a), np.sin(a)], 1)
+    g["tgt_onsurf"] = np.full(400, -1, np.int32)
+    q = 7
+    geo = Geometry(g, params_default(p_qbx=q, p_fmm=30, n_max=32))
+    geo.build()
+    out = geo.eval(kern, g["density"])
+    pts = np.nonzero(geo.association()[0] == 0)[0]
+    assert geo.info.list_size[3] > 100 and len(pts) > 100
+    f, s = np.longdouble, _strengths(g, g["density"])
+    use = s != 0
+    s, n, y = s[use].astype(f), g["up_n"][use].astype(f), g["up_xy"][use].astype(f)
+    z = (y[:, 0] + 1j * y[:, 1])[None] - (g["tgt_xy"][pts, 0].astype(f) + 1j * g["tgt_xy"][pts, 1].astype(f))[:, None]
+    t = (s * (n[:, 0] + 1j * n[:, 1]) / z).real if kern == "D" else s * np.log(np.abs(z))
+    tol = 70 * np.abs(s / z).sum(1) if kern == "D" else 3 * np.abs(s).sum() + 70 * np.abs(t).sum(1)
+    assert (np.abs(-2 * np.pi * out[pts] - t.sum(1)) <= tol * 2.0 ** -53).all()
+    c, r, _ = geo.centres()
+    sel = np.nonzero(np.repeat(np.repeat(g["panel_len"] > 0.05, 16), 2))[0][::7]
+    got = geo.qbx_coefficients()[sel] * r[sel, None] ** np.arange(q + 1)
+    geo.close()
+    ref, mag = _reference(g, kern, q, g["density"], sel, c, r)
+    if kern == "S":
+        got[:, 0], ref[:, 0] = got[:, 0].real, ref[:, 0].real
+        mag[:, 0] += 3 * np.abs(s).sum()
+    first = 1 if kern == "S" else 0
+    mag[:, first:] = np.maximum.accumulate(mag[:, first:], axis=1)
+    assert (np.abs(got - ref) <= 70 * 2.0 ** -53 * mag).all()
