@@ -149,3 +149,53 @@ def test_small_far_boxes(kern, levels):
     first = 1 if kern == "S" else 0
     mag[:, first:] = np.maximum.accumulate(mag[:, first:], axis=1)
     assert (np.abs(got - ref) <= 70 * 2.0 ** -53 * mag).all()
+
+
+@pytest.mark.parametrize("kern", ["S", "D"])
+@pytest.mark.parametrize("q", [4, 8, 13])
+def test_direct_sums_over_several_boxes(kern, q):
+    """A tree of one subdivision: several source ranges a box and no far lists, so that
+    the coefficients are the direct sums alone."""
+    from paper_1801_04070_gb300 import Geometry, params_default
+    g = _problem(16)
+    geo = Geometry(g, params_default(p_qbx=q, p_fmm=10, n_max=700))
+    geo.build()
+    assert geo.nbox > 1 and all(geo.info.list_size[i] == 0 for i in (1, 3, 5))
+    c, r, _ = geo.centres()
+    sel = np.arange(0, len(r), 5)
+    geo.eval(kern, g["density"])
+    got = geo.qbx_coefficients()[sel] * r[sel, None] ** np.arange(q + 1)
+    geo.close()
+    ref, mag = _reference(g, kern, q, g["density"], sel, c, r)
+    first = 1 if kern == "S" else 0
+    if kern == "S":
+        got[:, 0], ref[:, 0] = got[:, 0].real, ref[:, 0].real
+    mag[:, first:] = np.maximum.accumulate(mag[:, first:], axis=1)
+    tol = (q + 8 + np.log2(len(g["up_w"]))) * 2.0 ** -53 * mag
+    assert (np.abs(got - ref) <= tol).all(), (np.abs(got - ref) / tol).max()
+
+
+@pytest.mark.parametrize("p,q", [(17, 4), (18, 10), (20, 8), (30, 7), (15, 10)])
+@pytest.mark.parametrize("kern", ["S", "D"])
+def test_far_part_of_high_orders(kern, p, q):
+    """List 2, List 3 far and M2M in fixed point against FP64: the no-allocation
+    evaluation runs those in FP64 and the direct sums by the same kernel, so that what
+    differs are the translations alone, at every p_qbx within the bound of the other
+    List 2 and 3 comparisons."""
+    import ctypes as C
+
+    import torch
+    import workloads
+    from paper_1801_04070_gb300 import Geometry, _lib, params_default
+    g = workloads.small_grid(2, 2, 20, 4000, seed=p + q)
+    geo = Geometry(g, params_default(p_qbx=q, p_fmm=p, n_max=32, m2l=1))
+    geo.build()
+    assert geo.info.list_size[3] > 1000
+    dens = torch.tensor(g["density"], dtype=torch.float64, device="cuda")
+    a = torch.empty(geo.nt, dtype=torch.float64, device="cuda")
+    b = torch.empty_like(a)
+    geo.eval(kern, dens, a)
+    geo._check(geo.L.gq_eval_noalloc(geo._geom, _lib.KERNELS[kern], C.c_void_p(dens.data_ptr()), C.c_void_p(b.data_ptr())))
+    torch.cuda.synchronize()
+    geo.close()
+    assert (a - b).abs().max().item() <= 1e-13 * b.abs().max().item()
