@@ -606,14 +606,17 @@ def run_gpu(args, rank, world, local):
             e1.synchronize()
             step_ms.append(e0.elapsed_time(e1))
             eval_ms.append(st.ms_total)
-            stage_ms += np.array(st.ms_stage[:11])
     torch.cuda.synchronize()
     barrier(world)
     n1 = C.c_int64()
     chk(L.gq_context_launches(ctx, C.byref(n1)))
     launches = int(n1.value - n0.value)
     ms_step, value = replica_throughput(step_ms, nt, world, dev)
-    stage_ms /= args.steps
+    # each stage's own time: gq_eval's overlap
+    for _ in range(5):
+        flush.zero_()
+        chk(L.gq_eval_stages(geom, kern, d_mu.data_ptr(), d_out.data_ptr(), C.byref(st)))
+        stage_ms += np.array(st.ms_stage[:11]) / 5
 
     # ---- roofline of the dominant kernel (longest stage), FP64 ALU bound
     wrap = Geometry.__new__(Geometry)
@@ -784,6 +787,9 @@ def run_gpu(args, rank, world, local):
                     flush.zero_()
                     chk(L.gq_eval(sg, kern, d_mu.data_ptr(), d_out.data_ptr(), C.byref(sst)))
                     ms.append(sst.ms_total)
+                for _ in range(3):   # each stage's own time
+                    flush.zero_()
+                    chk(L.gq_eval_stages(sg, kern, d_mu.data_ptr(), d_out.data_ptr(), C.byref(sst)))
                     sms += np.array(sst.ms_stage[:11]) / 3
                 rp = params_default()
                 chk(L.gq_geometry_params(sg, C.byref(rp)))
@@ -835,6 +841,7 @@ def run_gpu(args, rank, world, local):
                 flush.zero_()
                 chk(L.gq_eval(sg, kern, d_mu.data_ptr(), d_out.data_ptr(), C.byref(sst)))
                 ems.append(sst.ms_total)
+            chk(L.gq_eval_stages(sg, kern, d_mu.data_ptr(), d_out.data_ptr(), C.byref(sst)))   # each stage's own time
             gh = Geometry.__new__(Geometry)
             gh.L, gh._ctx, gh._geom, gh.nt = L, ctx, sg, nt
             ti = TreeInfo()

@@ -194,9 +194,10 @@ typedef struct {
                                  4 L2L, 5 direct to centres (Lists 1, 3 close, 4 close),
                                  6 direct to point targets, 7 List 3 far to centres,
                                  8 List 3 far to point targets, 9 L2QBXL + L2P,
-                                 10 final QBX evaluation, 11 unused.  5 and 6 run on the
-                                 context's stream beside the others: the times of the
-                                 two sides overlap */
+                                 10 final QBX evaluation, 11 unused.  In gq_eval 5 and 6
+                                 (and often 7 and 8) run on the context's stream beside
+                                 the others: the times of the two sides overlap
+                                 (gq_eval_stages: each stage's own) */
 } gq_stats;
 
 /* Tree and list sizes after gq_build. */
@@ -255,6 +256,11 @@ gq_status gq_build(gq_geom *g);
  * density_base: [npanels*nb] density at base nodes (host or device).
  * out: [ntargets] potential values (host or device).  stats may be NULL. */
 gq_status gq_eval(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats);
+
+/* gq_eval with its stages one after another on the context's stream: the same
+ * values, and in `stats` (required) each stage's own time, where gq_eval's
+ * overlap.  For measurements. */
+gq_status gq_eval_stages(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats);
 
 /* The layer-potential operator at the base nodes, as an integral equation
  * applies it (Sec. 1: the exterior Neumann problem leads to the second-kind

@@ -78,6 +78,7 @@ def lib():
             "gq_targets_set": (st, [vp, i32, vp, vp]),
             "gq_build": (st, [vp]),
             "gq_eval": (st, [vp, i32, vp, vp, C.POINTER(Stats)]),
+            "gq_eval_stages": (st, [vp, i32, vp, vp, C.POINTER(Stats)]),
             "gq_eval_noalloc": (st, [vp, i32, vp, vp]),
             "gq_apply": (st, [vp, i32, C.c_double, vp, vp]),
             "gq_gmres": (st, [vp, vp, C.c_double, i32, i32, vp, C.POINTER(i32), C.POINTER(C.c_double)]),

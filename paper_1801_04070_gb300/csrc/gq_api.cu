@@ -286,7 +286,8 @@ gq_status gq_build(gq_geom *g) {
     });
 }
 
-gq_status gq_eval(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats) {
+static gq_status eval_call(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats,
+                           bool in_order) {
     if (!g || !density_base || (!out && g->nt > 0)) return GQ_ERR_INVALID;
     if (kernel != GQ_S && kernel != GQ_D && kernel != GQ_SP) return GQ_ERR_INVALID;
     return guarded(g->ctx, [&] {
@@ -305,7 +306,7 @@ gq_status gq_eval(gq_geom *g, int kernel, const double *density_base, double *ou
             o = g->out_dev.p;
         }
         if (stats) memset(stats, 0, sizeof(*stats));
-        gq_eval_all(g, kernel, dens, o, stats);
+        gq_eval_all(g, kernel, dens, o, stats, nullptr, nullptr, in_order);
         if (!out_dev && g->nt) {
             GQ_CUDA(cudaMemcpyAsync(out, o, sizeof(double) * g->nt, cudaMemcpyDefault, st));
             GQ_CUDA(cudaStreamSynchronize(st));
@@ -316,6 +317,15 @@ gq_status gq_eval(gq_geom *g, int kernel, const double *density_base, double *ou
         }
         }
     });
+}
+
+gq_status gq_eval(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats) {
+    return eval_call(g, kernel, density_base, out, stats, false);
+}
+
+gq_status gq_eval_stages(gq_geom *g, int kernel, const double *density_base, double *out, gq_stats *stats) {
+    if (!stats) return GQ_ERR_INVALID;
+    return eval_call(g, kernel, density_base, out, stats, true);
 }
 
 gq_status gq_apply(gq_geom *g, int kernel, double identity, const double *mu, double *out) {

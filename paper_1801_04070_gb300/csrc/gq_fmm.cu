@@ -1945,12 +1945,13 @@ static EvalTables &get_tables(gq_geom *g) {
 }
 
 void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev, gq_stats *stt,
-                 const double *apply_identity, const EvalFar *far) {
+                 const double *apply_identity, const EvalFar *far, bool in_order) {
     // apply_identity != null: the operator at the base nodes (gq_apply); the
     // point-target stages are skipped and out_dev has one value per base node.
     // far != null: strengths and the FMM passes only, their parts of the QBX
     // coefficients and point potentials written to far->Q, far->pot (the
     // batched evaluation does the direct parts and the final sums itself).
+    // in_order: every stage on the context's stream (stage times for measurements).
     const bool at_base = apply_identity != nullptr;
     const bool fmm_only = far != nullptr;
     // The evaluation's own copies of the context, one per stream: the context itself
@@ -2008,14 +2009,14 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     // 0.43 ms, 35 ragged curves 2.15 -> 1.89, 1.05 M nodes 11.4 -> 10.3.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     GQ_CUDA(cudaStreamIsCapturing(st, &cap));
-    const cudaStream_t sf = fmm_only ? st : g->s2;
+    const cudaStream_t sf = fmm_only || in_order ? st : g->s2;
     // List 3 far needs only the multipoles: it follows the direct part on the
     // context's stream, so that a chain of M2L, L2L and Stage 8 is left (35 curves
     // 1.89 -> 1.73 ms).  Where the direct part is the longer of the two it follows
     // M2L and L2L instead (1.05 M nodes, mixed tier: 8.86 -> 8.70), and in a captured
     // graph of many evaluations (12 geometries x 8 densities 35 -> 26 ms).  Either way
     // Stage 8 adds to its sums.
-    const bool w_beside = !fmm_only && cap == cudaStreamCaptureStatusNone && g->nsrc < 800000;
+    const bool w_beside = sf != st && cap == cudaStreamCaptureStatusNone && g->nsrc < 800000;
     gq_ctx passes = *ctx;   // launches of the FMM passes
     passes.stream = sf;
 
