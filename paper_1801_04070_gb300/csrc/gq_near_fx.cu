@@ -3,21 +3,21 @@
 //
 // S: Q_0 = sum q log|w|, Q_m = -(1/m) sum q (r/w)^m; D: Q_m = sum (d/w) (r/w)^m,
 // w = y - c.  In FP64 this sum issues 62 FP64 instructions a pair at q = 8 and
-// holds the FP64 pipe 88 % busy; here four are left (w and |w|^2), and 1/|w|^2,
-// r/w, log|w|, the power recurrence and the sums run on the integer pipes.  At
-// q = 8 a pair of a warp issues 440 instructions, about 110 of them 32 x 32 bit
-// multiply-adds of four cycles, which with the other work of that pipe bound
-// the kernel.  1.05 M quadrature nodes, 142.5 M pairs, S, q = 8: 17.06 ms -> 3.3 ms;
+// holds the FP64 pipe 88 % busy; here 7 are left (four a pair for w and |w|^2, the
+// rest for the sums' conversions), and 1/|w|^2, r/w, log|w|, the power recurrence and
+// the sums run on the integer pipes.  At q = 8 a pair costs 501 instructions of a lane
+// (idle lanes of the last round included), 210 of them on the pipe of the 32 x 32 bit
+// multiply-adds, which bounds the kernel: 70 % busy with 38 % of the warps resident.
+// 1.05 M quadrature nodes, 142.5 M pairs, S, q = 8: 17.06 ms -> 3.4 ms;
 // D on 0.14 M nodes: 2.59 -> 0.53 ms; q = 5 on one curve: 0.35 -> 0.14 ms.
 //
 // Formats (bits behind the binary point in brackets): u = r/w [62], t_m = q u^m
 // [60] with the strengths scaled to at most 1/2, products rounded at 2^-60.
 // |u| <= 1 when no source is inside the centre's disk; the loop records the
-// smallest |w|^2, and a centre that meets |u| > 1 + 1/64 is summed again.  While
-// (r/|w|)^q <= 2^4 (centres on the inner side of a sharp bend) that is with the
-// smallest |w| as its radius, and the sums are then scaled by (r/|w|)^m; above, the
-// sources inside are left out and their powers summed in FP64, since a scale that
-// holds them would leave the other sources' terms few bits or none.
+// smallest |w|^2, and a centre that meets |u| > 1 + 1/64 is summed again with the
+// smallest |w| as its radius; the sums are then scaled by (r/|w|)^m.  Where that would
+// raise the rounding above the terms (the sources inside are weak), they are left
+// out of a third sum and their powers summed in FP64.
 // Sums: 12 terms a lane (tiles of 384 sources), |t_m| < 0.65, stay below 2^63;
 // the warp's sum is taken at 2^-60 (2^-55 if the lanes' sums are that large).  Error against long double sums on the nodes
 // of a starfish grid (272 sources, q = 8, root mean square, in units of the
@@ -49,12 +49,14 @@ template <> struct FxStr<GQ_D> { typedef int4 T; };
 // FP64's: at n sources the sum's rounding, about sqrt(n) 2^-60 of that strength, has to
 // stay below 2^-53 of the sum of the terms' magnitudes, or the centre goes through
 // near_centre_fp64.  The bound on that sum in units of 2^-22 of the scale is
-// kFxWeak sqrt(n).  Errors against long double, q = 5 .. 16, one panel and another 2^k
-// times longer (host build of gq_fix.cuh): S equal at 2^11, 10 times FP64's at 2^14;
-// D at 2^8 and 2^11; this bound cuts at 2^9 and 2^7.  Panels of one length are 14 to 80
-// times above it.  Cost, 64 circles with panels graded over 2^20, q = 8, D: n_max 32 2.51 ->
-// 2.74 ms (all in FP64: 9.6), n_max 256 and 16 nodes a panel, where nearly all centres
-// mix 2^9 and more, 5.0 -> 18.3 (17.1).
+// kFxWeak sqrt(n), half of it for S.  Errors against long double, q = 5 .. 16, one panel
+// and another 2^k times longer (host build of gq_fix.cuh, root mean square): S equal to
+// FP64's at 2^11, 10 times at 2^14; D at 2^8 and 2^11; the bounds cut at 2^10 and 2^7.
+// Panels of one length are 28 to 160 (D 14 to 50) times above them; a tile of far
+// sources alone can fall below (S with D's bound: one leaf of 8,192 sources 1.41 -> 1.70
+// ms).  Cost, 64 circles with panels graded over 2^20, q = 8, D: n_max 32 2.51 ->
+// 2.68 ms (all in FP64: 9.6), n_max 256 and 16 nodes a panel, where nearly all centres
+// mix 2^9 and more, 5.0 -> 18.2 (17.1).
 constexpr float kFxWeak = 107021.0f;   // 2^21 at 384 sources
 
 __device__ __forceinline__ int fx_second(int2) { return 0; }
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
             bool any;
             const int qe = fx_stage<KERNEL>(E, R, v0, v1, sy, sq, ssum, smax, any);
             const bool scaled = qe > 0;
-            const float amin = any ? kFxWeak * sqrtf((float)n) : 0.0f;
+            const float amin = any ? (KERNEL == GQ_D ? kFxWeak : 0.5f * kFxWeak) * sqrtf((float)n) : 0.0f;
             for (int c = cb + w; c < ce; c += kFxWarps) {
                 const double2 cz = E.sc_xy[c];
                 const double rc = E.sc_r[c];
@@ -322,35 +324,39 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
                     nmax = __reduce_max_sync(0xffffffffu, nmax);
                 };
                 if (!slow) {
+                    bool inside;   // a source inside the disk, |u|^2 > 1 + 1/32
                     for (;;) {
                         sweep(std::false_type{});
-                        // a source inside the disk, |u|^2 > 1 + 1/32
                         const double wmin2 = __hiloint2double((int)nmin, 0);
-                        if (n == 0 || re != rc || !(rc * rc > wmin2 * (1.0 + 1.0 / 32))) break;
-                        if (rc * rc * exp2f(-8.0f / qc) <= wmin2) {
-                            re = sqrt(wmin2);
-                            continue;
-                        }
-                        nlim = (unsigned)(fx_bits(rc * rc * (32.0 / 33)) >> 32) + 1;
-                        sweep(std::true_type{});
-                        break;
+                        inside = n > 0 && rc * rc > wmin2 * (1.0 + 1.0 / 32);
+                        if (!inside || re != rc || (nmin >> 20) < 128) break;
+                        re = sqrt(wmin2);
                     }
-                    // |w|^2 a normal number far from the range's ends, the logarithms below 14
-                    const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20), er = fx_expo(fx_bits(re));
-                    slow = n > 0 && (emin < 128 || emax > 1920 || er < 128 || er > 1920 ||
-                                     (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40)));
-                    // the centre's terms weak beside the tile's scale (kFxWeak)
-                    const float a = (float)__reduce_add_sync(0xffffffffu, am >> 6);
-                    if (!slow && !(a >= amin)) slow = true;
-                    else if (!slow && re != rc) {
-                        // the rounding grows as (rc/re)^m: either the first order or the last has to stand above it
-                        unsigned aq = 0;
+                    float a = (float)__reduce_add_sync(0xffffffffu, am >> 6);
+                    if (inside) {
+                        // The sums are scaled by (rc/re)^m and their rounding with them: either the
+                        // last order (of the sources at re) or the first has to stand above it.
+                        bool held = false;
+                        if (re != rc) {
+                            unsigned aq = 0;
 #pragma unroll
-                        for (int m = 1; m <= QQ; ++m)
-                            if (m == qc) aq = abs((int)(acc[2 * m] >> 32)) + abs((int)(acc[2 * m + 1] >> 32));
-                        const float g = powf((float)(rc / re), (float)(qc - 1));
-                        slow = a < amin * g && !((float)__reduce_add_sync(0xffffffffu, aq >> 6) >= amin);
+                            for (int m = 1; m <= QQ; ++m)
+                                if (m == qc) aq = abs((int)(acc[2 * m] >> 32)) + abs((int)(acc[2 * m + 1] >> 32));
+                            held = (float)__reduce_add_sync(0xffffffffu, aq >> 6) >= amin ||
+                                   a >= amin * powf((float)(rc / re), (float)(qc - 1));
+                        }
+                        if (!held) {   // once more without the powers of the sources inside
+                            re = rc;
+                            nlim = (unsigned)(fx_bits(rc * rc * (32.0 / 33)) >> 32) + 1;
+                            sweep(std::true_type{});
+                            a = (float)__reduce_add_sync(0xffffffffu, am >> 6);
+                        }
                     }
+                    // |w|^2 a normal number far from the range's ends, the logarithms below 14, the
+                    // terms not weak beside the tile's scale (kFxWeak)
+                    const int emin = (int)(nmin >> 20), emax = (int)(nmax >> 20), er = fx_expo(fx_bits(re));
+                    slow = n > 0 && (emin < 128 || emax > 1920 || er < 128 || er > 1920 || (re == rc && !(a >= amin)) ||
+                                     (KERNEL != GQ_D && (emax - eref > 40 || eref - emin > 40)));
                 }
                 if (slow) {
                     near_centre_fp64<KERNEL, QQ < 9 ? QQ + 1 : 9>(E, R, v0, v1, cz, rc, QQ, qc, kAllSources, dst, first);
@@ -418,12 +424,13 @@ __global__ void __launch_bounds__(kNearThreads, fx_min_blocks(QQ)) k_near_centre
 // Potential at the point targets for S, sum q log|t - y| (coincident sources
 // skipped): a block per target box, a warp per target, lanes stride over the
 // staged sources; |w|^2 in FP64, logarithm, products and sums in fixed point.  The
-// FP64 pipe bounds it (83 % busy with 11.6 instructions a pair of a warp, at ten
-// targets and 70 sources a box): four a pair are |w|^2, so the conversions of
-// a target's sum wait in the lanes until 32 targets are converted by one
-// instruction, and the strengths' sum is formed once a tile.  Resident
-// blocks over several boxes, no staging, a warp a box or several targets a warp
-// were slower.  0.86 M point targets: 1.37 (FP64) -> 1.11 -> 0.78 ms.
+// FP64 pipe bounds it (79 % busy with 7.5 instructions a pair, at ten targets and 70
+// sources a box, which fill three rounds of a warp to three quarters): four are
+// |w|^2, so the conversions of a target's sum wait in the lanes until 32 targets are
+// converted by one instruction, and the strengths' sum is formed once a tile (11.6
+// instructions and 83 % before).  Resident blocks over several boxes, no staging, a
+// warp a box or several targets a warp were slower.  0.86 M point targets: 1.37 (FP64)
+// -> 1.11 -> 0.73 ms.  For D the point targets stay with the FP64 k_near_points.
 __global__ void __launch_bounds__(kNearThreads) k_near_points_fx(EvalView E, const int *__restrict__ work,
                                                                  double *__restrict__ pot) {
     __shared__ NearRanges R;
