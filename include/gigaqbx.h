@@ -81,7 +81,12 @@ enum { GQ_S = 0, GQ_D = 1, GQ_SP = 2 };
  *                 those of List 3 far that the tensor cores do not take, and
  *                 M2M run in 64-bit fixed point on the integer pipes (58 to
  *                 62 fraction bits, inputs and sums at shared exponents),
- *                 the rest in FP64 or as stated at m2l.
+ *                 the rest in FP64 or as stated at m2l.  Where a shared
+ *                 exponent would cost a direct sum digits (sources well
+ *                 inside a centre's disk, panels of very different length in
+ *                 one box) it runs in FP64.  A strength that is infinite or
+ *                 NaN, or a sum that overflows, makes the whole far field of
+ *                 its boxes NaN.
  *                 GQ_PREC_MIXED: a tier chosen from eps.
  *                 eps >= 5e-6: the direct interactions (Lists 1, 3 close,
  *                 4 close to centres and to point targets) and the List 3

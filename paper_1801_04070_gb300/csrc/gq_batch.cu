@@ -1,10 +1,8 @@
 // gq_batch.cu -- batched evaluation of many independent geometries and many
 // densities per geometry by one CUDA-graph launch.
 //
-// Each geometry's evaluations form one branch of the graph: the near-field QBX
-// coefficients of all its densities together (gq_eval_multi), then the rest of
-// the evaluation one density after another (they share the geometry's
-// expansion buffers); branches are
+// Each geometry's evaluations form one branch of the graph, one density after
+// another (they share the geometry's buffers); branches are
 // spread over S streams, largest first onto the least loaded stream, so small
 // problems run concurrently and fill the GPU.  The graph is captured once per
 // (kernel, densities, pointer set) and replayed afterwards.  S is chosen by an
@@ -86,16 +84,12 @@ void save_cache_file() {
     fclose(f);
 }
 
-// the ndens densities of one geometry (consecutive arrays), the direct part of
-// their QBX coefficients formed together (gq_eval_multi)
+// the ndens densities of one geometry (consecutive arrays), one after another: the
+// fixed-point direct sums of four densities cost less than forming the FP64 pair
+// geometry once for all four did
 void eval_densities(gq_geom *g, int kernel, int ndens, const double *dens, double *out) {
-    std::vector<const double *> d(ndens);
-    std::vector<double *> o(ndens);
-    for (int j = 0; j < ndens; ++j) {
-        d[j] = dens + (size_t)j * g->nbase;
-        o[j] = out + (size_t)j * g->nt;
-    }
-    gq_eval_multi(g, kernel, ndens, d.data(), o.data());
+    for (int j = 0; j < ndens; ++j)
+        gq_eval_all(g, kernel, dens + (size_t)j * g->nbase, out + (size_t)j * g->nt, nullptr);
 }
 
 // work estimate used to balance branches: quadrature nodes + targets + boxes

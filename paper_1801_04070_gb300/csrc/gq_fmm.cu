@@ -2012,10 +2012,13 @@ void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev
     const cudaStream_t sf = fmm_only || in_order ? st : g->s2;
     // List 3 far needs only the multipoles: it follows the direct part on the
     // context's stream, so that a chain of M2L, L2L and Stage 8 is left (35 curves
-    // 1.89 -> 1.73 ms).  Where the direct part is the longer of the two it follows
-    // M2L and L2L instead (1.05 M nodes, mixed tier: 8.86 -> 8.70), and in a captured
-    // graph of many evaluations (12 geometries x 8 densities 35 -> 26 ms).  Either way
-    // Stage 8 adds to its sums.
+    // 1.89 -> 1.73 ms).  Large problems, whose passes fill the SMs by themselves, put it
+    // after M2L and L2L instead.  The line lies between sizes measured both ways
+    // (beside -> after, ms): q 8, p 15 0.33 M nodes 3.19 -> 3.31, 0.59 M 5.16 -> 5.10,
+    // 0.80 M 6.84 -> 6.50, 1.05 M 8.69 -> 8.16; q 7, p 30 0.59 M 6.13 -> 6.17, 1.05 M
+    // 9.95 -> 9.24; mixed tier, q 4, p 19, 1.05 M 6.79 -> 6.34.  In a captured graph of
+    // many evaluations it follows too (12 geometries x 8 densities 35 -> 26 ms).
+    // Either way Stage 8 adds to its sums.
     const bool w_beside = sf != st && cap == cudaStreamCaptureStatusNone && g->nsrc < 800000;
     gq_ctx passes = *ctx;   // launches of the FMM passes
     passes.stream = sf;
@@ -2556,13 +2559,6 @@ int gq_bplan_error(gq_bplan *P) {
     GQ_CUDA(cudaMemsetAsync(P->err.p, 0, sizeof(int), st));
     GQ_CUDA(cudaStreamSynchronize(st));
     return h;
-}
-
-// Several densities on one geometry, one after another: the fixed-point direct
-// sums of four densities cost less than forming the FP64 pair geometry once for
-// all four did.
-void gq_eval_multi(gq_geom *g, int kernel, int nd, const double *const *dens, double *const *out) {
-    for (int d = 0; d < nd; ++d) gq_eval_all(g, kernel, dens[d], out[d], nullptr);
 }
 
 void gq_export_qbx_impl(gq_geom *g, double *host) {

@@ -235,7 +235,6 @@ struct EvalFar {
 void gq_eval_all(gq_geom *g, int kernel, const double *dens_dev, double *out_dev, gq_stats *st,
                  const double *apply_identity = nullptr, const EvalFar *far = nullptr,
                  bool in_order = false);                                                   // gq_fmm.cu
-void gq_eval_multi(gq_geom *g, int kernel, int nd, const double *const *dens, double *const *out);
 void gq_export_qbx_impl(gq_geom *g, double *host);  // gq_fmm.cu
 double gq_probe_fma(gq_ctx *ctx, int what);         // gq_probe.cu
 void gq_probe_math_impl(gq_ctx *ctx, int fn, int n, const double *x_dev, double *y_dev);

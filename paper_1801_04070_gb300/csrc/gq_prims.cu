@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kRsSmallThreads) k_rs_small(K *keys, int *vals
     __shared__ int run[W][kRsDigits];
     __shared__ int wtot[kRsDigits / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int per = ((n + W - 1) / W + 31) & ~31, i0 = min(n, w * per), i1 = min(n, i0 + per);   // per <= 32 items
+    const int per = ((n + W - 1) / W + 31) & ~31, i0 = min(n, w * per), i1 = min(n, i0 + per);   // per <= 32 kRsSmallItems
     const unsigned lt = (1u << lane) - 1u;
     for (int ps = 0; ps < passes; ++ps) {
         const int shift = ps * kRsBits;
