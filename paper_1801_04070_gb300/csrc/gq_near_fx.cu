@@ -5,9 +5,9 @@
 // w = y - c.  In FP64 this sum issues 62 FP64 instructions a pair at q = 8 and
 // holds the FP64 pipe 88 % busy; here 7 are left (four a pair for w and |w|^2, the
 // rest for the sums' conversions), and 1/|w|^2, r/w, log|w|, the power recurrence and
-// the sums run on the integer pipes.  At q = 8 a pair costs 501 instructions of a lane
-// (idle lanes of the last round included), 210 of them on the pipe of the 32 x 32 bit
-// multiply-adds, which bounds the kernel: 70 % busy with 38 % of the warps resident.
+// the sums run on the integer pipes.  At q = 8 a pair costs 505 instructions of a lane
+// (idle lanes of the last round included), 211 of them on the pipe of the 32 x 32 bit
+// multiply-adds, which bounds the kernel: 69 % busy with 38 % of the warps resident.
 // 1.05 M quadrature nodes, 142.5 M pairs, S, q = 8: 17.06 ms -> 3.4 ms;
 // D on 0.14 M nodes: 2.59 -> 0.53 ms; q = 5 on one curve: 0.35 -> 0.14 ms.
 //
